@@ -12,11 +12,11 @@
 
 namespace k2d {
 
-using ClassS = SizeClass<5, 2, 1, 1>;
-using ClassM = SizeClass<6, 3, 2, 2>;
-using ClassL = SizeClass<12, 4, 6, 2>;
+using ClassS = SizeClass<5, 2, 1, 1, 12>;
+using ClassM = SizeClass<6, 3, 2, 2, 16>;
+using ClassL = SizeClass<12, 4, 6, 2, 20>;
 
-constexpr int kMaxSlots = 8192;      // resident scene groups a launch may use (bounds the overflow scratch)
+constexpr int kMaxSlots = 8192;      // bounds the overflow scratch: room for this many slots of the batched contact solve
 constexpr size_t kCtrlBytes = 4096;  // control block at the start of the state buffer: 8 x uint64 counters, the work queue words at
                                      // kQueueOffset, the counting sort's words (2 x 256 + 1) at kSortOffset
 constexpr size_t kSortOffset = 1024;
@@ -28,8 +28,8 @@ constexpr int kChunkSteps = K2D_CHUNK_STEPS;       // steps per work item when t
 
 // run-time view of a size class
 struct ClassInfo {
-    int id, P, C, N, J, T, NPP, NPC, NCC, NPAIRS, NSLOTS, MASKW;
-    int LV_WORDS, ST_WORDS, SCRATCH_WORDS, PTAB_WORDS;
+    int id, P, C, N, J, T, NPP, NPC, NCC, NPAIRS, NSLOTS;
+    int LV_WORDS, ST_WORDS, SCRATCH_WORDS, SCRATCH_WORDS_BATCHED;
     int LV_X, LV_IM, LV_II, LV_FR, LV_RE, LV_FLAGS, LV_DENS, LV_RAD, LV_PVX, LV_PVY, LV_PNX, LV_PNY, LV_ELEN, LV_JOINT, LV_THR, LV_MASK, LV_GB;
     int ST_JACC, ST_META, ST_WARM;
 };
@@ -37,8 +37,8 @@ template <class SC>
 static ClassInfo make_info(int id) {
     ClassInfo c{};
     c.id = id; c.P = SC::P; c.C = SC::C; c.N = SC::N; c.J = SC::J; c.T = SC::T;
-    c.NPP = SC::NPP; c.NPC = SC::NPC; c.NCC = SC::NCC; c.NPAIRS = SC::NPAIRS; c.NSLOTS = SC::NSLOTS; c.MASKW = SC::MASKW;
-    c.LV_WORDS = SC::LV_WORDS; c.ST_WORDS = SC::ST_WORDS; c.SCRATCH_WORDS = SC::SCRATCH_WORDS; c.PTAB_WORDS = SC::PTAB_WORDS;
+    c.NPP = SC::NPP; c.NPC = SC::NPC; c.NCC = SC::NCC; c.NPAIRS = SC::NPAIRS; c.NSLOTS = SC::NSLOTS;
+    c.LV_WORDS = SC::LV_WORDS; c.ST_WORDS = SC::ST_WORDS; c.SCRATCH_WORDS = SC::SCRATCH_WORDS; c.SCRATCH_WORDS_BATCHED = SC::SCRATCH_WORDS_BATCHED;
     c.LV_X = SC::LV_X; c.LV_IM = SC::LV_IM; c.LV_II = SC::LV_II; c.LV_FR = SC::LV_FR; c.LV_RE = SC::LV_RE; c.LV_FLAGS = SC::LV_FLAGS;
     c.LV_DENS = SC::LV_DENS; c.LV_RAD = SC::LV_RAD; c.LV_PVX = SC::LV_PVX; c.LV_PVY = SC::LV_PVY; c.LV_PNX = SC::LV_PNX; c.LV_PNY = SC::LV_PNY;
     c.LV_ELEN = SC::LV_ELEN; c.LV_JOINT = SC::LV_JOINT; c.LV_THR = SC::LV_THR; c.LV_MASK = SC::LV_MASK; c.LV_GB = SC::LV_GB;
@@ -116,12 +116,14 @@ struct BufLayout { size_t ids_off, chunks_off, env_off, scratch_off, total; int 
 static BufLayout buffer_layout(const k2d_config *cfg, const ClassInfo &ci) {
     BufLayout b{};
     // every scene group of a launch can end up stepping an env, so the scratch covers whole blocks (up to 16 groups each)
-    b.slots = ((cfg->n_envs < kMaxSlots ? cfg->n_envs : kMaxSlots) + 15) / 16 * 16;
+    const size_t slots = ((cfg->n_envs < kMaxSlots ? cfg->n_envs : kMaxSlots) + 15) / 16 * 16;
+    // the sequential contact solve needs less per scene group, so the same memory serves more groups
+    b.slots = cfg->solver_batch > 0 ? (int)slots : (int)(slots * ci.SCRATCH_WORDS_BATCHED / ci.SCRATCH_WORDS);
     b.ids_off = kCtrlBytes;
     b.chunks_off = align_up(b.ids_off + (size_t)cfg->n_envs * 4, 256);
     b.env_off = align_up(b.chunks_off + (size_t)cfg->n_envs * 4, 256);
     b.scratch_off = align_up(b.env_off + (size_t)cfg->n_envs * ci.ST_WORDS * 4, 256);
-    b.total = align_up(b.scratch_off + (size_t)b.slots * ci.SCRATCH_WORDS * 4, 256);
+    b.total = align_up(b.scratch_off + slots * ci.SCRATCH_WORDS_BATCHED * 4, 256);
     return b;
 }
 
@@ -261,39 +263,46 @@ static int pack_level(const k2d_config *cfg, const ClassInfo &ci, const k2d_leve
             bool jn = false;
             for (auto &pr : joined) jn = jn || (pr.first == a && pr.second == b) || (pr.first == b && pr.second == a);
             if (jn) continue;
-            const int p = pair_index(ci.P, ci.C, a, b);
-            w[ci.LV_MASK + (p >> 5)] |= 1u << (p & 31);
+            w[ci.LV_MASK + a] |= 1u << b;
         }
     return K2D_OK;
 }
 
+// The block sizes a handle's step kernel can run in: one block per SM of LARGE threads, one of MID (where four scenes share a
+// warp; the same as LARGE elsewhere), or small blocks.
+template <class SC, int G>
+struct StepBlocks {
+    static constexpr int LARGE = step_block_threads<SC, G>(), MID = G == 8 && LARGE > 384 ? 384 : LARGE;
+};
+template <class SC, int G, class F>
+static cudaError_t with_step_kernel(int block_threads, F f) {
+    using B = StepBlocks<SC, G>;
+    if (block_threads == kSmallBlock) return f(k2d_step_kernel<SC, G, kSmallBlock>);
+    if (B::MID != B::LARGE && block_threads == B::MID) return f(k2d_step_kernel<SC, G, B::MID>);
+    return f(k2d_step_kernel<SC, G, B::LARGE>);
+}
 template <class SC, int G>
 static cudaError_t launch_step(const k2d_state *s, const StepParams &prm) {
-    constexpr int LARGE = step_block_threads<SC, G>();
-    if (s->large_block) k2d_step_kernel<SC, G, LARGE><<<s->grid, LARGE, s->smem_bytes, s->stream>>>(prm);
-    else k2d_step_kernel<SC, G, kSmallBlock><<<s->grid, kSmallBlock, s->smem_bytes, s->stream>>>(prm);
-    return cudaGetLastError();
+    return with_step_kernel<SC, G>(s->block_threads, [&](auto *kernel) {
+        kernel<<<s->grid, s->block_threads, s->smem_bytes, s->stream>>>(prm);
+        return cudaGetLastError();
+    });
 }
 // Launch shape of the step kernel for this handle.  With enough envs to give every scene group of the device one, the kernel
 // runs as one block per SM whose warps step in lockstep per scheduler; with fewer, as small blocks spread over all SMs.
 template <class SC, int G>
 static cudaError_t setup_step(k2d_state *s, int num_sms) {
-    constexpr int LARGE = step_block_threads<SC, G>();
-    s->large_block = LARGE > kSmallBlock && s->cfg.n_envs >= num_sms * (LARGE / G) && s->slots >= num_sms * (LARGE / G);
-    const int threads = s->large_block ? LARGE : kSmallBlock, GPB = threads / G;
+    using B = StepBlocks<SC, G>;
+    auto filled = [&](int threads) { return s->cfg.n_envs >= num_sms * (threads / G) && s->slots >= num_sms * (threads / G); };
+    const int threads = filled(B::LARGE) ? B::LARGE : filled(B::MID) ? B::MID : kSmallBlock, GPB = threads / G;
+    s->large_block = threads > kSmallBlock;
     s->block_threads = threads;
     s->smem_bytes = step_block_smem<SC, G>(threads);
-    cudaError_t err;
     int per_sm = 0;
-    if (s->large_block) {
-        err = cudaFuncSetAttribute(k2d_step_kernel<SC, G, LARGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s->smem_bytes);
-        if (err != cudaSuccess) return err;
-        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k2d_step_kernel<SC, G, LARGE>, threads, s->smem_bytes);
-    } else {
-        err = cudaFuncSetAttribute(k2d_step_kernel<SC, G, kSmallBlock>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s->smem_bytes);
-        if (err != cudaSuccess) return err;
-        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k2d_step_kernel<SC, G, kSmallBlock>, threads, s->smem_bytes);
-    }
+    cudaError_t err = with_step_kernel<SC, G>(threads, [&](auto *kernel) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s->smem_bytes);
+        return e != cudaSuccess ? e : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, s->smem_bytes);
+    });
     if (err != cudaSuccess) return err;
     if (per_sm < 1) per_sm = 1;
     int grid = num_sms * per_sm;
@@ -393,7 +402,7 @@ static cudaError_t order_envs(k2d_state *s, StepParams &prm) {
 // does the observation image of the handle's scenes fit into the part of a scene's shared-memory region the step kernel can spare for it?
 template <class SC, int G>
 static bool obs_fits(const k2d_state *s) {
-    return SC::WVX + k2d_obs_floats(&s->cfg) <= region_words<SC, G>();
+    return obs_image_word<SC>() + k2d_obs_floats(&s->cfg) <= region_words<SC, G>();
 }
 
 }  // namespace k2d
@@ -487,12 +496,11 @@ int k2d_create(const k2d_config *cfg, void *dev_state_buf, void *dev_level_pool_
     cudaError_t err = cudaSetDevice(cfg->device);
     int num_sms = 0;
     if (err == cudaSuccess) err = cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, cfg->device);
-    // default lanes per scene: a warp per scene while the device has warps to spare (measured on B200: faster below
-    // about 48 envs per SM for the largest size class, 24 for the smaller ones), two scenes per warp beyond
-    // default lanes per scene: two scenes per warp once they fill the device's one-block-per-SM form (40 scenes per SM) with
-    // some to spare, one scene per warp below that (measured, env-steps/s with 16 against 32 lanes: L x 8192 132.8 M / 107.2 M,
-    // L x 6144 99.1 M / 103.3 M, L x 4096 70.3 M / 97.9 M, M x 4096 112.8 M / 143.3 M, S x 4096 147.7 M / 164.9 M)
-    if (err == cudaSuccess && !cfg->lanes_per_scene) s->G = (cfg->n_envs < (kLargeBlock / 16) * num_sms * 9 / 8) ? 32 : 16;
+    // default lanes per scene: four scenes per warp once they fill the device's one-block-per-SM form (48 scenes per SM), with
+    // fewer envs more lanes per scene, so that a step of a scene takes less time
+    if (err == cudaSuccess && !cfg->lanes_per_scene) s->G = cfg->n_envs >= 48 * num_sms ? 8 : cfg->n_envs >= 12 * num_sms ? 16 : 32;
+    // with few batches one of them can hold more manifolds than eight lanes
+    if (!cfg->lanes_per_scene && cfg->solver_batch > 0 && 4 * cfg->solver_batch > ci.NSLOTS && s->G < 16) s->G = 16;
     if (err == cudaSuccess) err = K2D_DISPATCH(setup_step, s, s, num_sms);
     if (err == cudaSuccess) err = cudaMemcpyAsync(s->dev_levels, s->host_levels.data(), s->host_levels.size() * 4, cudaMemcpyHostToDevice, s->stream);
     if (err == cudaSuccess) err = cudaStreamSynchronize(s->stream);
@@ -692,8 +700,7 @@ int k2d_level_info(const k2d_config *cfg, const k2d_level *host_level, float *ho
     if (host_collide)
         for (int a = 0; a < nN; ++a)
             for (int b = a + 1; b < nN; ++b) {
-                const int q = pair_index(ci.P, ci.C, internal(a), internal(b));
-                host_collide[pair_index(nP, nC, a, b)] = (uint8_t)((lv[ci.LV_MASK + (q >> 5)] >> (q & 31)) & 1u);
+                host_collide[pair_index(nP, nC, a, b)] = (uint8_t)((lv[ci.LV_MASK + internal(a)] >> internal(b)) & 1u);
             }
     return K2D_OK;
 }
@@ -757,7 +764,7 @@ int k2d_eval_sincos_tanh(const float *dev_x, int32_t n, float *dev_cos, float *d
 
 // ---- k2d_step for callers that cannot provide the overflow scratch: it lives in the library image.
 // One array per device that loads the library, held until the process exits.
-static __device__ __align__(256) uint32_t k2d_static_scratch[(size_t)K2D_STATIC_SCRATCH_MAX_ENVS * ClassL::SCRATCH_WORDS];
+static __device__ __align__(256) uint32_t k2d_static_scratch[(size_t)K2D_STATIC_SCRATCH_MAX_ENVS * ClassL::SCRATCH_WORDS_BATCHED];
 static std::mutex k2d_static_mutex;
 static uint32_t *k2d_static_ptr[64];     // device address of the array on each device, filled on first use
 
