@@ -238,6 +238,8 @@ static int pack_level(const k2d_config *cfg, const ClassInfo &ci, const k2d_leve
         jw[10] = L->joint_fixed[j] ? 1u : (L->joint_limited[j] ? 2u : 0u);
         joined.emplace_back(a, b);
     }
+    for (int q = 0; q < ci.N; ++q)      // friction coefficients whose squares overflow (the step then limits friction by comparisons)
+        if (is_active[q] && u2f(w[ci.LV_FR + q]) > 1.0e18f) w[ci.LV_GB] |= 1u << 27;
     w[ci.LV_GB] |= (uint32_t)std::min(joint_levels, 7) << 24;      // what the launch's env order sorts by (with the touching pairs)
     std::fill(body_level.begin(), body_level.end(), 0);
     for (int t = 0; t < nT; ++t) {
