@@ -498,9 +498,12 @@ int k2d_create(const k2d_config *cfg, void *dev_state_buf, void *dev_level_pool_
     cudaError_t err = cudaSetDevice(cfg->device);
     int num_sms = 0;
     if (err == cudaSuccess) err = cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, cfg->device);
-    // default lanes per scene: four scenes per warp once they fill the device's one-block-per-SM form (48 scenes per SM), with
-    // fewer envs more lanes per scene, so that a step of a scene takes less time
-    if (err == cudaSuccess && !cfg->lanes_per_scene) s->G = cfg->n_envs >= 48 * num_sms ? 8 : cfg->n_envs >= 12 * num_sms ? 16 : 32;
+    // Default lanes per scene: four scenes per warp from 32 scenes per SM on, which is what two scenes per warp in small blocks
+    // hold at once (us for two steps with 16 / 8 lanes: L x 4096 83.8 / 84.5, L x 6144 146 / 94, M x 4096 53.1 / 59.0, M x 6144
+    // 97 / 64, S x 4096 46.1 / 47.5, S x 6144 85 / 52); one scene per warp below 16 scenes per SM for the large size class, 7 for
+    // the smaller ones, whose few records fit into 16 lanes' registers (32 / 16 lanes: L x 2048 67.6 / 73.8, M x 1024
+    // 42.2 / 42.6, M x 2048 49.3 / 45.3, M x 512 39.1 / 40.9).
+    if (err == cudaSuccess && !cfg->lanes_per_scene) s->G = cfg->n_envs >= 32 * num_sms ? 8 : cfg->n_envs >= (ci.id == 2 ? 16 : 7) * num_sms ? 16 : 32;
     // with few batches one of them can hold more manifolds than eight lanes
     if (!cfg->lanes_per_scene && cfg->solver_batch > 0 && 4 * cfg->solver_batch > ci.NSLOTS && s->G < 16) s->G = 16;
     if (err == cudaSuccess) err = K2D_DISPATCH(setup_step, s, s, num_sms);
