@@ -270,6 +270,18 @@ static int pack_level(const k2d_config *cfg, const ClassInfo &ci, const k2d_leve
     return K2D_OK;
 }
 
+// Launches a kernel that begins with after_previous_kernel(): its blocks may take their places on the SMs while the kernel in
+// front of it in the stream is still running.
+template <class... P, class... A>
+static cudaError_t launch_after(void (*kernel)(P...), int grid, int threads, size_t smem, cudaStream_t stream, A... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3((unsigned)threads); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+    cfg.attrs = &attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
 // The block sizes a handle's step kernel can run in: one block per SM of LARGE threads, one of MID (where four scenes share a
 // warp; the same as LARGE elsewhere), or small blocks.
 template <class SC, int G>
@@ -286,8 +298,7 @@ static cudaError_t with_step_kernel(int block_threads, F f) {
 template <class SC, int G>
 static cudaError_t launch_step(const k2d_state *s, const StepParams &prm) {
     return with_step_kernel<SC, G>(s->block_threads, [&](auto *kernel) {
-        kernel<<<s->grid, s->block_threads, s->smem_bytes, s->stream>>>(prm);
-        return cudaGetLastError();
+        return launch_after(kernel, s->grid, s->block_threads, s->smem_bytes, s->stream, prm);
     });
 }
 // Launch shape of the step kernel for this handle.  With enough envs to give every scene group of the device one, the kernel
@@ -323,15 +334,13 @@ static cudaError_t launch_obs(const k2d_state *s, float *dev_obs) {
     const int epb = kObsEnvsPerBlock, grid = (c.n_envs + epb - 1) / epb;
     const int width = (c.n_polygons + c.n_circles) * 29 + c.n_joints * 2 * (11 + c.n_actions) + c.n_thrusters * 6;
     const size_t smem = sizeof(float) * epb * obs_image_stride(width, SC::N);
-    k2d_obs_kernel<SC><<<grid, kObsThreads, smem, s->stream>>>(s->dev_env, s->dev_levels, dev_obs, c.n_envs, c.n_actions, c.n_polygons,
-                                                              c.n_circles, c.n_joints, c.n_thrusters);
-    return cudaGetLastError();
+    return launch_after(k2d_obs_kernel<SC>, grid, kObsThreads, smem, s->stream, s->dev_env, s->dev_levels, dev_obs, c.n_envs, c.n_actions, c.n_polygons,
+                        c.n_circles, c.n_joints, c.n_thrusters);
 }
 
 template <class SC>
 static cudaError_t launch_render(const k2d_state *s, uint32_t *out) {
-    k2d_render_kernel<SC><<<s->cfg.n_envs, kRenderThreads, 0, s->stream>>>(s->dev_env, s->dev_levels, out, s->cfg.n_envs);
-    return cudaGetLastError();
+    return launch_after(k2d_render_kernel<SC>, s->cfg.n_envs, kRenderThreads, 0, s->stream, s->dev_env, s->dev_levels, out, s->cfg.n_envs);
 }
 
 // Kernel arguments of one k2d_step launch.  With more envs than resident scene groups the launch is cut
@@ -372,9 +381,9 @@ constexpr int kOrderMinSteps = 8, kOrderShortLaunches = 16;
 template <class SC>
 static cudaError_t launch_order(const k2d_state *s) {
     const int n = s->cfg.n_envs, grid = (n + kOrderThreads - 1) / kOrderThreads;
-    k2d_order_count_kernel<SC><<<grid, kOrderThreads, 0, s->stream>>>(s->dev_env, s->dev_levels, s->dev_sort, n, s->cfg.n_levels);
-    k2d_order_place_kernel<SC><<<grid, kOrderThreads, 0, s->stream>>>(s->dev_env, s->dev_levels, s->dev_sort, s->dev_ids, n, s->cfg.n_levels);
-    return cudaGetLastError();
+    const cudaError_t err = launch_after(k2d_order_count_kernel<SC>, grid, kOrderThreads, 0, s->stream, s->dev_env, s->dev_levels, s->dev_sort, n, s->cfg.n_levels);
+    if (err != cudaSuccess) return err;
+    return launch_after(k2d_order_place_kernel<SC>, grid, kOrderThreads, 0, s->stream, s->dev_env, s->dev_levels, s->dev_sort, s->dev_ids, n, s->cfg.n_levels);
 }
 // with one scene per warp and small blocks nothing runs in lockstep, and with no more envs than groups every group gets one env anyway
 static bool uses_order(const k2d_state *s) {
