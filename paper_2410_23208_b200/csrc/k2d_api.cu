@@ -1,5 +1,6 @@
 // k2d_api.cu -- host side of the C ABI declared in include/k2d.h: validation, level build (mass
 // properties, collision mask, constraint levels), buffer layout, kernel launches.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -12,9 +13,16 @@
 
 namespace k2d {
 
+// The last number is how many contact pair records of a scene live in shared memory.  With eight lanes per scene, where 64
+// scenes share an SM's shared memory, it is what fits (about one L scene in a thousand has more than 20 touching pairs); with
+// fewer scenes per SM there is room for every record a schedule can hold, and the launch does not wait for the one scene whose
+// last records are in global memory.
 using ClassS = SizeClass<5, 2, 1, 1, 12>;
 using ClassM = SizeClass<6, 3, 2, 2, 16>;
 using ClassL = SizeClass<12, 4, 6, 2, 20>;
+using ClassSRoomy = SizeClass<5, 2, 1, 1, 21>;
+using ClassMRoomy = SizeClass<6, 3, 2, 2, kSchedRecords>;
+using ClassLRoomy = SizeClass<12, 4, 6, 2, kSchedRecords>;
 
 constexpr int kMaxSlots = 8192;      // bounds the overflow scratch: room for this many slots of the batched contact solve
 constexpr size_t kCtrlBytes = 4096;  // control block at the start of the state buffer: 8 x uint64 counters, the work queue words at
@@ -136,7 +144,10 @@ static int pack_level(const k2d_config *cfg, const ClassInfo &ci, const k2d_leve
     const int nP = cfg->n_polygons, nC = cfg->n_circles, nN = nP + nC, nJ = cfg->n_joints, nT = cfg->n_thrusters;
     std::memset(w, 0, sizeof(uint32_t) * ci.LV_WORDS);
     auto internal = [&](int i) { return i < nP ? i : ci.P + (i - nP); };
-    std::vector<int> is_static(ci.N, 1), is_active(ci.N, 0);
+    // (a pool of a thousand levels is packed while the caller waits: no allocations, sets of shapes as bit masks)
+    int is_static[K2D_MAX_SHAPES], is_active[K2D_MAX_SHAPES];
+    std::fill(is_static, is_static + K2D_MAX_SHAPES, 1);
+    std::fill(is_active, is_active + K2D_MAX_SHAPES, 0);
     for (int i = 0; i < nN; ++i) {
         const int q = internal(i);
         const float pose[6] = { L->pos[i][0], L->pos[i][1], L->angle[i], L->vel[i][0], L->vel[i][1], L->angvel[i] };
@@ -207,8 +218,8 @@ static int pack_level(const k2d_config *cfg, const ClassInfo &ci, const k2d_leve
     }
     // joints: "on" when both shapes exist and at least one can move; level = 1 + highest level of an earlier
     // joint sharing a movable shape (so lanes can run a level's joints at once and keep the joint order)
-    std::vector<int> body_level(ci.N, 0);
-    std::vector<std::pair<int, int>> joined;
+    int body_level[K2D_MAX_SHAPES] = {};
+    uint32_t joined[K2D_MAX_SHAPES] = {};      // per shape: the shapes it is joined to
     int joint_levels = 0;
     for (int j = 0; j < nJ; ++j) {
         uint32_t *jw = w + ci.LV_JOINT + kJointLevelWords * j;
@@ -236,12 +247,12 @@ static int pack_level(const k2d_config *cfg, const ClassInfo &ci, const k2d_leve
                 (((L->joint_fixed[j] || L->joint_limited[j]) ? 1u : 0u) << 31);
         for (int k = 0; k < 9; ++k) jw[1 + k] = f2u(v[k]);
         jw[10] = L->joint_fixed[j] ? 1u : (L->joint_limited[j] ? 2u : 0u);
-        joined.emplace_back(a, b);
+        joined[a] |= 1u << b; joined[b] |= 1u << a;
     }
     for (int q = 0; q < ci.N; ++q)      // friction coefficients whose squares overflow (the step then limits friction by comparisons)
         if (is_active[q] && u2f(w[ci.LV_FR + q]) > 1.0e18f) w[ci.LV_GB] |= 1u << 27;
     w[ci.LV_GB] |= (uint32_t)std::min(joint_levels, 7) << 24;      // what the launch's env order sorts by (with the touching pairs)
-    std::fill(body_level.begin(), body_level.end(), 0);
+    std::fill(body_level, body_level + K2D_MAX_SHAPES, 0);
     for (int t = 0; t < nT; ++t) {
         uint32_t *tw = w + ci.LV_THR + 8 * t;
         if (!L->thr_active[t]) continue;
@@ -259,14 +270,10 @@ static int pack_level(const k2d_config *cfg, const ClassInfo &ci, const k2d_leve
         tw[1] = f2u(v[0]); tw[2] = f2u(v[1]); tw[3] = f2u((float)std::cos(phi)); tw[4] = f2u((float)std::sin(phi)); tw[5] = f2u(v[3]);
     }
     // which pairs may collide: both shapes present, not both fixated, not joined (paper: joined shapes do not collide)
+    uint32_t active = 0u, movable = 0u;
+    for (int q = 0; q < ci.N; ++q) { if (is_active[q]) active |= 1u << q; if (!is_static[q]) movable |= 1u << q; }
     for (int a = 0; a < ci.N; ++a)
-        for (int b = a + 1; b < ci.N; ++b) {
-            if (!is_active[a] || !is_active[b] || (is_static[a] && is_static[b])) continue;
-            bool jn = false;
-            for (auto &pr : joined) jn = jn || (pr.first == a && pr.second == b) || (pr.first == b && pr.second == a);
-            if (jn) continue;
-            w[ci.LV_MASK + a] |= 1u << b;
-        }
+        if (is_active[a]) w[ci.LV_MASK + a] = active & (is_static[a] ? movable : ~0u) & ~joined[a] & ~((2u << a) - 1u);
     return K2D_OK;
 }
 
@@ -406,9 +413,9 @@ static cudaError_t order_envs(k2d_state *s, StepParams &prm) {
 }
 
 #define K2D_DISPATCH(FN, s, ...)                                                                      \
-    ((s)->ci.id == 0 ? ((s)->G == 32 ? FN<ClassS, 32>(__VA_ARGS__) : (s)->G == 16 ? FN<ClassS, 16>(__VA_ARGS__) : FN<ClassS, 8>(__VA_ARGS__)) \
-   : (s)->ci.id == 1 ? ((s)->G == 32 ? FN<ClassM, 32>(__VA_ARGS__) : (s)->G == 16 ? FN<ClassM, 16>(__VA_ARGS__) : FN<ClassM, 8>(__VA_ARGS__)) \
-                     : ((s)->G == 32 ? FN<ClassL, 32>(__VA_ARGS__) : (s)->G == 16 ? FN<ClassL, 16>(__VA_ARGS__) : FN<ClassL, 8>(__VA_ARGS__)))
+    ((s)->ci.id == 0 ? ((s)->G == 32 ? FN<ClassSRoomy, 32>(__VA_ARGS__) : (s)->G == 16 ? FN<ClassS, 16>(__VA_ARGS__) : FN<ClassS, 8>(__VA_ARGS__)) \
+   : (s)->ci.id == 1 ? ((s)->G == 32 ? FN<ClassMRoomy, 32>(__VA_ARGS__) : (s)->G == 16 ? FN<ClassM, 16>(__VA_ARGS__) : FN<ClassM, 8>(__VA_ARGS__)) \
+                     : ((s)->G == 32 ? FN<ClassLRoomy, 32>(__VA_ARGS__) : (s)->G == 16 ? FN<ClassLRoomy, 16>(__VA_ARGS__) : FN<ClassL, 8>(__VA_ARGS__)))
 
 // does the observation image of the handle's scenes fit into the part of a scene's shared-memory region the step kernel can spare for it?
 template <class SC, int G>

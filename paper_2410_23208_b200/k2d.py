@@ -363,14 +363,15 @@ def noop_outcomes(levels: dict, n_steps: int, device: int = 0, chunk: int = 32, 
     n = levels["pos"].shape[0]
     env = Env(levels, n, device=device, auto_reset=RESET_NONE, max_fused_steps=chunk, **cfg_kw)
     zeros = torch.zeros((chunk, n, env.n_actions), dtype=torch.float32, device=env.device)
-    rs, ds = [], []
+    # all launches are enqueued before the host waits for the first result
+    reward = torch.empty((n_steps, n), dtype=torch.float32, device=env.device)
+    done = torch.empty((n_steps, n), dtype=torch.uint8, device=env.device)
     for s0 in range(0, n_steps, chunk):
         k = min(chunk, n_steps - s0)
-        r, d = env.step(zeros[:k])
-        rs.append(r.cpu().numpy())
-        ds.append(d.cpu().numpy())
+        env.step(zeros[:k], reward[s0:s0 + k], done[s0:s0 + k])
+    r, d = reward.cpu().numpy(), done.cpu().numpy()
     env.close()
-    return first_outcomes(np.concatenate(rs), np.concatenate(ds))
+    return first_outcomes(r, d)
 
 
 def shard_envs(n_envs_total: int, rank: int, world_size: int):
