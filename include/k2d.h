@@ -108,7 +108,7 @@ typedef struct k2d_config {
     uint64_t seed;                 /* seed of the K2D_RESET_POOL hash                           */
     int64_t env_offset;            /* global index of env 0 (sharding over several GPUs)        */
     int32_t device;                /* CUDA device ordinal                                       */
-    int32_t lanes_per_scene;       /* 0 = library default (32 for few envs, else 16); or 8, 16, 32 */
+    int32_t lanes_per_scene;       /* 0 = library default (32 for few envs, 8 for many); or 8, 16, 32 */
     int32_t solver_batch;          /* 0 = contacts solved one after the other (default); B > 0 = the paper's batched solve, see below */
     int32_t reserved;              /* 0 */
     void *cuda_stream;             /* cudaStream_t of the caller (NULL = default stream)        */
@@ -277,7 +277,7 @@ int k2d_resident_groups(const k2d_state *s);
 int k2d_lanes_per_scene(const k2d_state *s);
 int k2d_step_launches(const k2d_state *s, int32_t n_steps);
 /* Test aid: the work items ((run of 8 steps, env) pairs) that one ticket of a launch's work queue stands for: the scene
- * groups of the warps that step in lockstep (10 for L scenes on a full device). */
+ * groups of the warps that step in lockstep (16 on a full device with the default lanes per scene). */
 int k2d_items_per_ticket(const k2d_state *s);
 
 /* Measurement aid.  In a library compiled with -DK2D_PHASE_CLOCKS the step kernel adds up, per phase of an environment
