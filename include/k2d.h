@@ -269,14 +269,14 @@ int k2d_trace_slots(const k2d_state *s);
 int k2d_is_checked_build(void);
 
 /* Host-side facts about a handle's launches.  k2d_resident_groups: scenes the device steps at once for this handle (with
- * more envs than that a launch goes through a work queue, and from one and a half times as many on it first sorts the envs
+ * more envs than that a launch goes through a work queue, and from 1.3 to 1.5 times as many on it first sorts the envs
  * by what their steps cost, in two small launches of its own; launches of fewer than 8 steps reuse that order 16 times).  k2d_lanes_per_scene: 8, 16 or 32.
  * k2d_step_launches: kernel launches that the next k2d_step, k2d_step_discrete or k2d_step_obs call with n_steps steps
  * makes (1 or 3; k2d_step_obs one more for scenes whose observation does not fit beside the scene in shared memory). */
 int k2d_resident_groups(const k2d_state *s);
 int k2d_lanes_per_scene(const k2d_state *s);
 int k2d_step_launches(const k2d_state *s, int32_t n_steps);
-/* Test aid: the work items ((run of 8 steps, env) pairs) that one ticket of a launch's work queue stands for: the scene
+/* Test aid: the work items ((run of steps, env) pairs) that one ticket of a launch's work queue stands for: the scene
  * groups of the warps that step in lockstep (16 on a full device with the default lanes per scene). */
 int k2d_items_per_ticket(const k2d_state *s);
 
@@ -289,7 +289,7 @@ int k2d_items_per_ticket(const k2d_state *s);
 #define K2D_PHASES 14
 int k2d_phase_cycles(k2d_state *s, uint64_t *host_cycles, int32_t n);
 
-/* Test aid.  With more envs than the device holds scene groups, k2d_step hands out runs of 8 steps of an env to whichever
+/* Test aid.  With more envs than the device holds scene groups, k2d_step hands out runs of 8 (or 4) steps of an env to whichever
  * group is free; a group that gets a later run of an env before the earlier one is back in memory polls for it, about
  * every 100 ns, at most `polls` times (default 2^24, a few seconds; values below 64 are raised to 64), then records
  * K2D_ERR_WAIT for k2d_status and gives up.  A small limit lets a test make that wait run out. */

@@ -350,8 +350,15 @@ static cudaError_t launch_render(const k2d_state *s, uint32_t *out) {
     return launch_after(k2d_render_kernel<SC>, s->cfg.n_envs, kRenderThreads, 0, s->stream, s->dev_env, s->dev_levels, out, s->cfg.n_envs);
 }
 
+// Steps per work item when there are more envs than resident scene groups.  With eight lanes per scene and less than one and a
+// half waves of envs the launch ends in a wave that is mostly empty; shorter items fill it better (us for 32 steps, items of
+// 8 / 4 steps: L x 10000 1545 / 1512, L x 12000 1703 / 1648, M x 12000 1110 / 1065; with more envs the loads of more items cost
+// as much: M x 16384 1291 / 1298, L x 131072 15.11 / 15.55 ms).
+static int chunk_steps(const k2d_state *s) {
+    return s->large_block && s->G == 8 && 2 * (long long)s->cfg.n_envs < 3 * (long long)s->groups ? kChunkSteps / 2 : kChunkSteps;
+}
 // Kernel arguments of one k2d_step launch.  With more envs than resident scene groups the launch is cut
-// into chunks of kChunkSteps steps, so that the groups can balance the work between them.
+// into chunks of that many steps, so that the groups can balance the work between them.
 static StepParams step_params(const k2d_state *s, const float *dev_actions, int n_steps, float *dev_reward, uint8_t *dev_done,
                               uint32_t *scratch, int discrete = 0) {
     const k2d_config &c = s->cfg;
@@ -368,10 +375,11 @@ static StepParams step_params(const k2d_state *s, const float *dev_actions, int 
         prm.n_batches = c.solver_batch > 0 ? (n_slots + c.solver_batch - 1) / c.solver_batch : 0;
         if (c.solver_batch > 0 && prm.n_batches < 1) prm.n_batches = 1;
     }
-    if (c.n_envs > s->groups && n_steps > kChunkSteps) {
-        const int n_chunks = (n_steps + kChunkSteps - 1) / kChunkSteps;
+    const int chunk = chunk_steps(s);
+    if (c.n_envs > s->groups && n_steps > chunk) {
+        const int n_chunks = (n_steps + chunk - 1) / chunk;
         if ((unsigned long long)c.n_envs * (unsigned long long)n_chunks + (unsigned long long)s->groups < 0xffffffffULL) {
-            prm.chunk_steps = kChunkSteps; prm.n_chunks = n_chunks;
+            prm.chunk_steps = chunk; prm.n_chunks = n_chunks;
         }
     }
     prm.solver_iters = c.solver_iters; prm.warm_start = c.warm_start; prm.auto_reset = c.auto_reset; prm.max_episode_steps = c.max_episode_steps;
@@ -394,9 +402,10 @@ static cudaError_t launch_order(const k2d_state *s) {
 }
 // with one scene per warp and small blocks nothing runs in lockstep, and with no more envs than groups every group gets one env anyway
 static bool uses_order(const k2d_state *s) {
-    // one block per SM: from one and a half waves of envs on (measured on L scenes, sorted against unsorted env-steps/s:
-    // 7400 envs 114.6 M / 123.6 M, 8192 132.1 M / 135.8 M, 9000 140.3 M / 137.6 M, 12000 152.9 M / 141.9 M, 16384 158.3 M / 146.8 M)
-    if (s->large_block) return 2 * (long long)s->cfg.n_envs > 3 * (long long)s->groups;
+    // one block per SM: with eight lanes per scene from four thirds of a wave of envs on (us for 32 steps, unsorted / sorted:
+    // L x 10000, 1.06 waves, 1512 / 1595, L x 12000 1648 / 1732, L x 14000 1798 / 1787, M x 14000 1222 / 1116, L x 16384
+    // 2099 / 2065, L x 131072 15980 / 15107), with more lanes from one and a half
+    if (s->large_block) return s->G == 8 ? 3 * (long long)s->cfg.n_envs > 4 * (long long)s->groups : 2 * (long long)s->cfg.n_envs > 3 * (long long)s->groups;
     return s->G < 32 && s->cfg.n_envs > s->groups;
 }
 // a short launch reuses the order of an earlier one (what an env's step costs changes slowly) and sorts again every
