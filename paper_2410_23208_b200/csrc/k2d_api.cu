@@ -106,7 +106,7 @@ struct k2d_state {
     unsigned long long *dev_counters;
     unsigned int *dev_queue, *dev_chunks, *dev_sort;
     int block_threads;   // threads per block of the step kernel for this handle
-    bool large_block;    // one block per SM, warps in lockstep per scheduler (enough envs to fill the device)
+    bool large_block;    // several warps per scheduler, in lockstep
     int order_age;       // launches since the envs were last sorted for the work queue (0: the order is not valid)
     int *dev_ids;
     uint32_t *dev_env, *dev_scratch, *dev_levels;
@@ -289,49 +289,49 @@ static cudaError_t launch_after(void (*kernel)(P...), int grid, int threads, siz
     cfg.attrs = &attr; cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
-// The block sizes a handle's step kernel can run in: one block per SM of LARGE threads, one of MID (where four scenes share a
-// warp; the same as LARGE elsewhere), or small blocks.
-template <class SC, int G>
-struct StepBlocks {
-    static constexpr int LARGE = step_block_threads<SC, G>(), MID = G == 8 && LARGE > 384 ? 384 : LARGE;
-};
-template <class SC, int G, class F>
+// calls f with the step kernel in blocks of block_threads threads (a multiple of kSmallBlock up to THREADS)
+template <class SC, int G, int THREADS, class F>
 static cudaError_t with_step_kernel(int block_threads, F f) {
-    using B = StepBlocks<SC, G>;
-    if (block_threads == kSmallBlock) return f(k2d_step_kernel<SC, G, kSmallBlock>);
-    if (B::MID != B::LARGE && block_threads == B::MID) return f(k2d_step_kernel<SC, G, B::MID>);
-    return f(k2d_step_kernel<SC, G, B::LARGE>);
+    if constexpr (THREADS > kSmallBlock) {
+        if (block_threads < THREADS) return with_step_kernel<SC, G, THREADS - kSmallBlock>(block_threads, f);
+    }
+    return f(k2d_step_kernel<SC, G, THREADS>);
 }
 template <class SC, int G>
 static cudaError_t launch_step(const k2d_state *s, const StepParams &prm) {
-    return with_step_kernel<SC, G>(s->block_threads, [&](auto *kernel) {
+    return with_step_kernel<SC, G, step_block_threads<SC, G>()>(s->block_threads, [&](auto *kernel) {
         return launch_after(kernel, s->grid, s->block_threads, s->smem_bytes, s->stream, prm);
     });
 }
-// Launch shape of the step kernel for this handle.  With enough envs to give every scene group of the device one, the kernel
-// runs as one block per SM whose warps step in lockstep per scheduler; with fewer, as small blocks spread over all SMs.
+// Launch shape of the step kernel for this handle: one block per SM, of the fewest threads that give every env a scene group (one
+// wave), or of the most threads, whose groups then take the envs from a queue.  In a launch of one wave a scratch slot belongs
+// to an env, in one of several to a scene group.
 template <class SC, int G>
 static cudaError_t setup_step(k2d_state *s, int num_sms) {
-    using B = StepBlocks<SC, G>;
-    auto filled = [&](int threads) { return s->cfg.n_envs >= num_sms * (threads / G) && s->slots >= num_sms * (threads / G); };
-    const int threads = filled(B::LARGE) ? B::LARGE : filled(B::MID) ? B::MID : kSmallBlock, GPB = threads / G;
+    const int n = s->cfg.n_envs;
+    auto capacity = [&](int t) { return num_sms * (t / G); };
+    int threads = kSmallBlock;
+    while (threads < step_block_threads<SC, G>() && capacity(threads) < n) threads += kSmallBlock;
+    if (capacity(threads) < n || n > s->slots)
+        while (threads > kSmallBlock && capacity(threads) > s->slots) threads -= kSmallBlock;
+    const int GPB = threads / G;
     s->large_block = threads > kSmallBlock;
     s->block_threads = threads;
     s->smem_bytes = step_block_smem<SC, G>(threads);
     int per_sm = 0;
-    cudaError_t err = with_step_kernel<SC, G>(threads, [&](auto *kernel) {
+    cudaError_t err = with_step_kernel<SC, G, step_block_threads<SC, G>()>(threads, [&](auto *kernel) {
         const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s->smem_bytes);
         return e != cudaSuccess ? e : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, s->smem_bytes);
     });
     if (err != cudaSuccess) return err;
-    if (per_sm < 1) per_sm = 1;
-    int grid = num_sms * per_sm;
-    const int need = (s->cfg.n_envs + GPB - 1) / GPB;
-    if (grid > need) grid = need;
-    if (grid * GPB > s->slots) grid = s->slots / GPB;
+    if (per_sm < 1) return cudaErrorInvalidConfiguration;
+    // the warps of a scheduler take per_batch envs together: no more blocks than that gives something to do
+    const int per_batch = (threads / 128) * (32 / G);
+    int grid = std::min(num_sms, (n + per_batch - 1) / per_batch);
+    if (grid * GPB < n && grid * GPB > s->slots) grid = s->slots / GPB;
     if (grid < 1) grid = 1;
     s->grid = grid;
-    s->groups = grid * GPB;
+    s->groups = std::min(grid * GPB, n);
     return cudaSuccess;
 }
 
@@ -814,7 +814,7 @@ int k2d_step_static_scratch(k2d_state *s, const float *dev_actions, int32_t n_st
     if (n_steps < 1 || n_steps > s->cfg.max_fused_steps) return K2D_ERR_STEPS;
     if (((uintptr_t)dev_actions & 3) || ((uintptr_t)dev_reward & 3)) return K2D_ERR_ALIGN;
     const k2d_config &c = s->cfg;
-    if (c.n_envs > K2D_STATIC_SCRATCH_MAX_ENVS || s->groups > K2D_STATIC_SCRATCH_MAX_ENVS || c.device >= 64) {
+    if (c.n_envs > K2D_STATIC_SCRATCH_MAX_ENVS || c.device >= 64) {
         std::fprintf(stderr, "k2d_step_static_scratch: n_envs = %d is beyond the built-in scratch (at most %d envs); use k2d_step\n",
                      c.n_envs, K2D_STATIC_SCRATCH_MAX_ENVS);
         return K2D_ERR_LIMIT;
@@ -832,7 +832,7 @@ int k2d_step_static_scratch(k2d_state *s, const float *dev_actions, int32_t n_st
         scratch = k2d_static_ptr[c.device];
     }
     const StepParams prm = step_params(s, dev_actions, n_steps, dev_reward, dev_done, scratch);
-    // a launch never has more scene groups than envs rounded up to a whole block, so the limit on n_envs bounds the scratch slots
+    // a scratch slot goes with an env, or with one of fewer groups than envs, so the limit on n_envs bounds the slots
     CUDA_OK(K2D_DISPATCH(launch_step, s, s, prm));
     return K2D_OK;
 }

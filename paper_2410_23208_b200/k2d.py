@@ -250,7 +250,7 @@ class Env:
         out = {}
         for name, shape in (("pos", (N, 2)), ("angle", (N,)), ("vel", (N, 2)), ("angvel", (N,)), ("acc", (S, 2)), ("jacc", (J, 3))):
             n = int(np.prod(shape))
-            out[name] = f[:, o:o + n].reshape((-1,) + shape).copy()
+            out[name] = f[:, o:o + n].reshape((raw.shape[0],) + shape).copy()
             o += n
         meta = raw[:, o:o + 4].view(np.int32)
         for k, name in enumerate(("step_count", "episode_count", "level_id", "status")):
