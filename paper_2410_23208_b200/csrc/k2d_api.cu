@@ -107,6 +107,7 @@ struct k2d_state {
     unsigned int *dev_queue, *dev_chunks, *dev_sort;
     int block_threads;   // threads per block of the step kernel for this handle
     bool large_block;    // several warps per scheduler, in lockstep
+    int apart_grid;      // blocks of a launch of one step in blocks of kSmallBlock threads (0: not used)
     int order_age;       // launches since the envs were last sorted for the work queue (0: the order is not valid)
     int *dev_ids;
     uint32_t *dev_env, *dev_scratch, *dev_levels;
@@ -289,6 +290,12 @@ static cudaError_t launch_after(void (*kernel)(P...), int grid, int threads, siz
     cfg.attrs = &attr; cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
+// A launch of one wave and one step whose block would take all registers of an SM (512 threads and more) runs in small blocks
+// instead, several to an SM, if those hold all envs at once: they can take their places while the kernels around them are still
+// running.  One step, without and with an observation behind it (us, one block / small blocks): S x 4096 28.2 / 25.6 and
+// 33.8 / 31.5, M x 4096 31.5 / 28.4 and 37.3 / 34.6, L x 2048 31.8 / 31.5 and 39.9 / 38.1; with smaller blocks it depends (L x 3000
+// 37.5 / 41.2), with two steps the lockstep is worth more (L x 4096 74.6 / 77.3).
+constexpr int kApartThreads = 512;
 // calls f with the step kernel in blocks of block_threads threads (a multiple of kSmallBlock up to THREADS)
 template <class SC, int G, int THREADS, class F>
 static cudaError_t with_step_kernel(int block_threads, F f) {
@@ -299,8 +306,10 @@ static cudaError_t with_step_kernel(int block_threads, F f) {
 }
 template <class SC, int G>
 static cudaError_t launch_step(const k2d_state *s, const StepParams &prm) {
-    return with_step_kernel<SC, G, step_block_threads<SC, G>()>(s->block_threads, [&](auto *kernel) {
-        return launch_after(kernel, s->grid, s->block_threads, s->smem_bytes, s->stream, prm);
+    const bool apart = prm.n_steps == 1 && s->apart_grid > 0;
+    const int grid = apart ? s->apart_grid : s->grid, threads = apart ? kSmallBlock : s->block_threads;
+    return with_step_kernel<SC, G, step_block_threads<SC, G>()>(threads, [&](auto *kernel) {
+        return launch_after(kernel, grid, threads, apart ? step_block_smem<SC, G>(kSmallBlock) : s->smem_bytes, s->stream, prm);
     });
 }
 // Launch shape of the step kernel for this handle: one block per SM, of the fewest threads that give every env a scene group (one
@@ -330,6 +339,17 @@ static cudaError_t setup_step(k2d_state *s, int num_sms) {
     int grid = std::min(num_sms, (n + per_batch - 1) / per_batch);
     if (grid * GPB < n && grid * GPB > s->slots) grid = s->slots / GPB;
     if (grid < 1) grid = 1;
+    if (threads == kSmallBlock) grid = std::min(grid, (n + GPB - 1) / GPB);
+    s->apart_grid = 0;
+    if (threads >= kApartThreads && grid * GPB >= n) {
+        int small_per_sm = 0;
+        const size_t smem = step_block_smem<SC, G>(kSmallBlock);
+        err = cudaFuncSetAttribute(k2d_step_kernel<SC, G, kSmallBlock>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (err == cudaSuccess) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&small_per_sm, k2d_step_kernel<SC, G, kSmallBlock>, kSmallBlock, smem);
+        if (err != cudaSuccess) return err;
+        const int need = (n + kSmallBlock / G - 1) / (kSmallBlock / G);
+        if (need <= num_sms * small_per_sm) s->apart_grid = need;
+    }
     s->grid = grid;
     s->groups = std::min(grid * GPB, n);
     return cudaSuccess;
@@ -400,7 +420,7 @@ static cudaError_t launch_order(const k2d_state *s) {
     if (err != cudaSuccess) return err;
     return launch_after(k2d_order_place_kernel<SC>, grid, kOrderThreads, 0, s->stream, s->dev_env, s->dev_levels, s->dev_sort, s->dev_ids, n, s->cfg.n_levels);
 }
-// with one scene per warp and small blocks nothing runs in lockstep, and with no more envs than groups every group gets one env anyway
+// with no more envs than groups every group gets one env anyway
 static bool uses_order(const k2d_state *s) {
     // one block per SM: with eight lanes per scene from four thirds of a wave of envs on (us for 32 steps, unsorted / sorted:
     // L x 10000, 1.06 waves, 1512 / 1595, L x 12000 1648 / 1732, L x 14000 1798 / 1787, M x 14000 1222 / 1116, L x 16384
@@ -523,11 +543,11 @@ int k2d_create(const k2d_config *cfg, void *dev_state_buf, void *dev_level_pool_
     cudaError_t err = cudaSetDevice(cfg->device);
     int num_sms = 0;
     if (err == cudaSuccess) err = cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, cfg->device);
-    // Default lanes per scene: four scenes per warp from 32 scenes per SM on, which is what two scenes per warp in small blocks
-    // hold at once (us for two steps with 16 / 8 lanes: L x 4096 83.8 / 84.5, L x 6144 146 / 94, M x 4096 53.1 / 59.0, M x 6144
-    // 97 / 64, S x 4096 46.1 / 47.5, S x 6144 85 / 52); one scene per warp below 16 scenes per SM for the large size class, 7 for
-    // the smaller ones, whose few records fit into 16 lanes' registers (32 / 16 lanes: L x 2048 67.6 / 73.8, M x 1024
-    // 42.2 / 42.6, M x 2048 49.3 / 45.3, M x 512 39.1 / 40.9).
+    // Default lanes per scene.  Eight from 32 scenes per SM on, which is where a block of 512 threads of two scenes per warp is
+    // full (us for 32 steps with 16 / 8 lanes: L x 4700 1091 / 1127, L x 5300 1373 / 1200, M x 4700 674 / 750, M x 5300 849 / 806,
+    // S x 4700 584 / 610, S x 5300 699 / 649); one scene per warp up to 16 scenes per SM for the large size class (32 / 16 lanes:
+    // L x 2048 826 / 890, L x 2500 1103 / 967) and up to 7 for the smaller ones, whose few records fit into 16 lanes' registers
+    // (M x 560 510 / 516, M x 1500 564 / 560, M x 2048 624 / 568).
     if (err == cudaSuccess && !cfg->lanes_per_scene) s->G = cfg->n_envs >= 32 * num_sms ? 8 : cfg->n_envs >= (ci.id == 2 ? 16 : 7) * num_sms ? 16 : 32;
     // with few batches one of them can hold more manifolds than eight lanes
     if (!cfg->lanes_per_scene && cfg->solver_batch > 0 && 4 * cfg->solver_batch > ci.NSLOTS && s->G < 16) s->G = 16;

@@ -93,3 +93,28 @@ def test_env_counts_around_the_launch_shapes(n_envs):
     (r, d), (rr, dr) = parity.step_both(env, ref, act[9:], chunk=1, n_threads=8)
     err, exact = parity.errors(env, ref)
     assert exact, err
+
+
+@pytest.mark.parametrize("size,n_envs,lanes", [("S", 593, 32), ("S", 1183, 32), ("S", 2368, 16), ("M", 2369, 16), ("L", 1185, 32), ("L", 4735, 16), ("S", 4737, 8), ("L", 2663, 0)])
+def test_block_sizes_of_launches_of_one_wave(size, n_envs, lanes):
+    # one block per SM of 128, 256, 384 or 512 threads, envs on either side of a full device; one step at a time (small blocks
+    # where the block would fill an SM) and several
+    lv = scenes.make_levels(size, 48, 66, static_prob=0.1)
+    lv["pos"][:8, 1:, 0] *= 0.3          # a few piles, whose records reach the scratch slots
+    env, ref = parity.make_pair(lv, n_envs, lanes_per_scene=lanes, auto_reset=2, max_episode_steps=6, seed=66)
+    assert env.resident_groups == n_envs
+    act = scenes.make_actions(9, n_envs, env.n_actions, 66)
+    (r, d), (rr, dr) = parity.step_both(env, ref, act[:2], chunk=1, n_threads=8)
+    assert np.array_equal(r, rr) and np.array_equal(d, dr)
+    (r, d), (rr, dr) = parity.step_both(env, ref, act[2:], n_threads=8)
+    err, exact = parity.errors(env, ref)
+    assert exact and np.array_equal(r, rr) and np.array_equal(d, dr), err
+
+
+def test_state_of_scenes_without_joints():
+    dims = scenes.SceneDims(6, 0, 0, 1)
+    lv = scenes.make_levels(dims, 8, 67)
+    env, ref = parity.make_pair(lv, 8)
+    _exact(env, ref, scenes.make_actions(5, 8, env.n_actions, 67))
+    env.set_state(env.get_state())
+    _exact(env, ref, scenes.make_actions(5, 8, env.n_actions, 68))
