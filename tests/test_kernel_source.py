@@ -1,0 +1,53 @@
+"""CPU-side checks of the kernel source: rules that the compiler does not enforce and that no output shows when they are broken."""
+import os
+import re
+
+from paper_2410_23208_b200 import build
+
+KERNELS = os.path.join(build.HERE, "csrc", "k2d_kernels.cuh")
+
+
+def _source():
+    """the kernel source without its comments"""
+    text = re.sub(r"/\*.*?\*/", "", open(KERNELS).read(), flags=re.S)
+    return re.sub(r"//[^\n]*", "", text)
+
+
+def _arguments(text, call):
+    """(position, argument text) of every call of the function"""
+    for m in re.finditer(r"\b%s\(" % re.escape(call), text):
+        depth, i = 1, m.end()
+        while depth:
+            depth += {"(": 1, ")": -1}.get(text[i], 0)
+            i += 1
+        yield m.start(), text[m.end():i - 1]
+
+
+def _base(expression):
+    """the pointer an address expression starts from"""
+    inner = re.sub(r"reinterpret_cast<[^>]*>\(", "", expression)
+    return re.match(r"[\s(]*([A-Za-z_][\w.]*)", inner).group(1)
+
+
+def test_read_only_cache_loads_read_nothing_but_the_level_pool():
+    # A load through the read-only cache (__ldg) is defined only for words that nobody writes while the kernel is on the
+    # device, and a kernel launched ahead of its turn is on the device while the kernel in front of it still writes.  The
+    # level pool, written once by the host, is the only input that qualifies.
+    text = _source()
+
+    def in_pool(name, at):
+        if name in ("levels", "prm.levels"):
+            return True
+        if "." in name:
+            return False
+        # the definition in force: the last one before the use, a variable's or a level record handed in as a parameter
+        found = list(re.finditer(r"\*\s*%s( = [^;]*;|\s*[,)])" % re.escape(name), text[:at]))
+        assert found, name
+        d = found[-1]
+        return name == "lv" if not d.group(1).startswith(" =") else in_pool(_base(d.group(1)[3:]), d.start())
+
+    calls = list(_arguments(text, "__ldg"))
+    assert len(calls) > 10
+    for at, argument in calls:
+        assert in_pool(_base(argument), at), f"__ldg({argument}) does not read the level pool"
+    assert not re.search(r"ld\.global\.nc|__restrict__", text)
