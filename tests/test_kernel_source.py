@@ -23,6 +23,21 @@ def _arguments(text, call):
         yield m.start(), text[m.end():i - 1]
 
 
+def _without_calls(text, name):
+    """the text without the calls name<...>(...), arguments included"""
+    out, at = [], 0
+    for m in re.finditer(r"\b%s<\w+>\(" % re.escape(name), text):
+        if m.start() < at:
+            continue
+        depth, i = 1, m.end()
+        while depth:
+            depth += {"(": 1, ")": -1}.get(text[i], 0)
+            i += 1
+        out.append(text[at:m.start()])
+        at = i
+    return "".join(out) + text[at:]
+
+
 def _base(expression):
     """the pointer an address expression starts from"""
     inner = re.sub(r"reinterpret_cast<[^>]*>\(", "", expression)
@@ -51,3 +66,12 @@ def test_read_only_cache_loads_read_nothing_but_the_level_pool():
     for at, argument in calls:
         assert in_pool(_base(argument), at), f"__ldg({argument}) does not read the level pool"
     assert not re.search(r"ld\.global\.nc|__restrict__", text)
+
+
+def test_every_body_index_of_a_contact_pair_goes_through_the_index_check():
+    # the two 5-bit body fields of a pair word ("ab", alone, in an array of a lane's words or in a record) and the 4-bit ones of
+    # a survivor code; the checked build replaces an index out of range, a raw field would be used as it is
+    text = _without_calls(_source(), "ck_idx")
+    raw = re.findall(r"[^;{}]*\b(?:ab(?:\[i\])?|code)(?: >> \d+\))? & (?:15|31)\b[^;{}]*;", text)
+    assert not raw, raw
+    assert len(re.findall(r"ck_idx<CK_BODY>", _source())) > 20
