@@ -362,12 +362,12 @@ static cudaError_t launch_obs(const k2d_state *s, float *dev_obs) {
     const int width = (c.n_polygons + c.n_circles) * 29 + c.n_joints * 2 * (11 + c.n_actions) + c.n_thrusters * 6;
     const size_t smem = sizeof(float) * epb * obs_image_stride(width, SC::N);
     return launch_after(k2d_obs_kernel<SC>, grid, kObsThreads, smem, s->stream, s->dev_env, s->dev_levels, dev_obs, c.n_envs, c.n_actions, c.n_polygons,
-                        c.n_circles, c.n_joints, c.n_thrusters);
+                        c.n_circles, c.n_joints, c.n_thrusters, c.n_levels);
 }
 
 template <class SC>
 static cudaError_t launch_render(const k2d_state *s, uint32_t *out) {
-    return launch_after(k2d_render_kernel<SC>, s->cfg.n_envs, kRenderThreads, 0, s->stream, s->dev_env, s->dev_levels, out, s->cfg.n_envs);
+    return launch_after(k2d_render_kernel<SC>, s->cfg.n_envs, kRenderThreads, 0, s->stream, s->dev_env, s->dev_levels, out, s->cfg.n_envs, s->cfg.n_levels);
 }
 
 // Steps per work item when there are more envs than resident scene groups.  With eight lanes per scene and less than one and a

@@ -94,6 +94,54 @@ def test_a_bad_count_in_the_state_record_is_caught_and_redirected():
     assert env.status()[3] == 4 * n_envs
 
 
+# S scenes: words of a level record (joint, thruster, the dense reward's shapes) and of a state record (level id), in bytes from
+# the start of their buffer, and what is planted there
+PLANTED = {
+    "joint": ("level_buf", 4 * 188, 0xff, 200),
+    "thruster": ("level_buf", 4 * 200, 0xff, 200),
+    "first green shape": ("level_buf", 4 * 215, 0xff, 250),
+    "level id": ("state_buf", 4096 + 512 + 4 * (6 * 7 + 3 + 2), 0xffffffff, 99999),
+}
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("what,call", [(w, c) for w in ("joint", "thruster", "level id") for c in ("step", "step_obs", "obs")] +
+                         [("first green shape", "step"), ("level id", "render"), ("level id", "reset inside the step")])
+def test_a_bad_index_in_a_level_or_state_record_is_caught_and_redirected(what, call):
+    # checked build only: the word is wrong in the caller's own buffer, every use of it is compared with its limit and redirected
+    import torch
+    n_envs = 8
+    lv = scenes.make_levels("S", n_envs, 3)
+    env = k2d.Env(lv, n_envs, checked=True, dense_kappa=0.1, auto_reset=1, max_episode_steps=2 if "reset" in call else 0)
+    assert (env.cfg.n_polygons, env.cfg.n_circles, env.cfg.n_joints, env.cfg.n_thrusters) == (5, 2, 1, 1)
+    act = torch.zeros((4, n_envs, env.n_actions), device="cuda")
+
+    def run():
+        if call == "step_obs":
+            env.step_obs(act)
+        elif call in ("obs", "render"):
+            getattr(env, call)()
+        else:
+            env.step(act)
+        torch.cuda.synchronize()
+
+    run()
+    env.status()
+    name, at, mask, value = PLANTED[what]
+    word = getattr(env, name)[at:at + 4].view(torch.int32)
+    good = int(word[0])
+    new = (good & 0xffffffff & ~mask) | value
+    word[0] = new - (1 << 32) if new >= 1 << 31 else new
+    torch.cuda.synchronize()
+    run()
+    with pytest.raises(k2d.K2DError, match="index check"):
+        env.status()
+    word[0] = good
+    env.reset()
+    run()
+    env.status()
+
+
 # ---------------------------------------------------------------- the build that counts cycles per phase of a step
 def test_phase_clock_library_builds_and_the_plain_library_refuses_the_call():
     from paper_2410_23208_b200 import build

@@ -68,10 +68,19 @@ def test_read_only_cache_loads_read_nothing_but_the_level_pool():
     assert not re.search(r"ld\.global\.nc|__restrict__", text)
 
 
-def test_every_body_index_of_a_contact_pair_goes_through_the_index_check():
-    # the two 5-bit body fields of a pair word ("ab", alone, in an array of a lane's words or in a record) and the 4-bit ones of
-    # a survivor code; the checked build replaces an index out of range, a raw field would be used as it is
+def test_every_body_index_goes_through_the_index_check():
+    # the body fields of a contact pair's word ("ab": alone, in an array of a lane's words or in a record), of a survivor code, of
+    # a joint's or thruster's word and of the dense reward's shapes; the checked build replaces an index out of range, a raw
+    # field would be used as it is.  An action binding is no index here: it is compared with the number of channels.
     text = _without_calls(_source(), "ck_idx")
-    raw = re.findall(r"[^;{}]*\b(?:ab(?:\[i\])?|code)(?: >> \d+\))? & (?:15|31)\b[^;{}]*;", text)
-    assert not raw, raw
-    assert len(re.findall(r"ck_idx<CK_BODY>", _source())) > 20
+    raw = re.findall(r"[^;{}]*\b(?:ab(?:\[i\])?|code|jab|jw0|tp|gb)(?: >> \d+\))? & (?:15|31|255)u?\b[^;{}]*;", text)
+    assert not [r for r in raw if "bind = " not in r], raw
+    assert len(re.findall(r"ck_idx<CK_BODY>", _source())) > 30
+
+
+def test_every_level_id_goes_through_the_index_check():
+    text = _without_calls(_source(), "ck_idx")
+    text = re.sub(r"enum \{ META_STEP[^}]*\}", "", text)
+    text = re.sub(r"\w+\[SC::META \+ META_LEVEL\] = [^;]*;", "", text)                # stores
+    text = re.sub(r"min\(__ldcg\(st \+ SC::ST_META \+ META_LEVEL\), [^;]*;", "", text)      # limited in every build
+    assert not re.findall(r"[^;{}]*META_LEVEL[^;{}]*;", text)
