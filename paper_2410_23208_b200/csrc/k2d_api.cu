@@ -410,8 +410,9 @@ static StepParams step_params(const k2d_state *s, const float *dev_actions, int 
 }
 
 // Launches of at least kOrderMinSteps steps with two or more scenes per warp and more envs than the device holds scene groups
-// first sort the envs by what their steps cost (see k2d_order_count_kernel); the order lives in the words that k2d_reset uses
-// for the level ids, free between resets.
+// first sort the envs by what their steps cost (see k2d_order_count_kernel); the order lives in the words through which k2d_reset
+// hands over level ids, and k2d_reset leaves them as the order by index: a launch recorded into a graph while it reused an
+// order finds a permutation there whatever was called since.
 constexpr int kOrderMinSteps = 8, kOrderShortLaunches = 16;
 template <class SC>
 static cudaError_t launch_order(const k2d_state *s) {
@@ -574,10 +575,10 @@ int k2d_reset(k2d_state *s, const int32_t *host_level_ids) {
 #endif
     CUDA_OK(cudaMemsetAsync(s->dev_chunks, 0, (size_t)E * 4, s->stream));
     if (host_level_ids) CUDA_OK(cudaMemcpyAsync(s->dev_ids, host_level_ids, (size_t)E * 4, cudaMemcpyHostToDevice, s->stream));
-    const int *ids = host_level_ids ? s->dev_ids : nullptr;
-    if (s->ci.id == 0) k2d_reset_kernel<ClassS><<<E, 64, 0, s->stream>>>(s->dev_env, s->dev_levels, ids, E, s->cfg.n_levels);
-    else if (s->ci.id == 1) k2d_reset_kernel<ClassM><<<E, 64, 0, s->stream>>>(s->dev_env, s->dev_levels, ids, E, s->cfg.n_levels);
-    else k2d_reset_kernel<ClassL><<<E, 64, 0, s->stream>>>(s->dev_env, s->dev_levels, ids, E, s->cfg.n_levels);
+    const int ids_given = host_level_ids ? 1 : 0;
+    if (s->ci.id == 0) k2d_reset_kernel<ClassS><<<E, 64, 0, s->stream>>>(s->dev_env, s->dev_levels, s->dev_ids, ids_given, E, s->cfg.n_levels);
+    else if (s->ci.id == 1) k2d_reset_kernel<ClassM><<<E, 64, 0, s->stream>>>(s->dev_env, s->dev_levels, s->dev_ids, ids_given, E, s->cfg.n_levels);
+    else k2d_reset_kernel<ClassL><<<E, 64, 0, s->stream>>>(s->dev_env, s->dev_levels, s->dev_ids, ids_given, E, s->cfg.n_levels);
     CUDA_OK(cudaGetLastError());
     CUDA_OK(cudaStreamSynchronize(s->stream));
     return K2D_OK;
