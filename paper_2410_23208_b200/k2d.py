@@ -141,7 +141,11 @@ def make_config(levels: dict, n_envs: int, **kw) -> Config:
 
 
 class Env:
-    """n_envs scenes on one CUDA device, stepped by the library."""
+    """n_envs scenes on one CUDA device, stepped by the library.
+
+    All work goes to ``stream`` (default: the stream that is current when the Env is made).  What the Env allocates belongs to
+    that stream; tensors handed in from another stream have to be ready when the call is made and must not be freed before
+    ``stream`` has passed it."""
 
     def __init__(self, levels: dict, n_envs: int, device: int = 0, stream=None, checked: bool = False, phase_clocks: bool = False, **cfg_kw):
         import torch
@@ -158,9 +162,7 @@ class Env:
         lb = self.lib.k2d_level_pool_bytes(C.byref(self.cfg))
         if sb == 0 or lb == 0:
             raise K2DError("invalid config")
-        with torch.cuda.device(self.device):
-            self.state_buf = torch.empty(sb, dtype=torch.uint8, device=self.device)
-            self.level_buf = torch.empty(lb, dtype=torch.uint8, device=self.device)
+        self.state_buf, self.level_buf = self._empty((sb,), torch.uint8), self._empty((lb,), torch.uint8)
         packed = pack_levels(levels)
         h = C.c_void_p()
         _check(self.lib.k2d_create(C.byref(self.cfg), self.state_buf.data_ptr(), self.level_buf.data_ptr(),
@@ -169,6 +171,23 @@ class Env:
         self.obs_floats = self.lib.k2d_obs_floats(C.byref(self.cfg))
         self.canonical_words = self.lib.k2d_canonical_words(C.byref(self.cfg))
         self._trace = None
+
+    def _empty(self, shape, dtype):
+        """Device memory that the library's stream may write at once.  The allocator hands a freed block out again as soon as
+        nothing that is still to come on the block's own stream can use it, so the block has to be the library's stream's; the
+        caller's stream, if that is another, may go on using it until it is freed."""
+        torch = self.torch
+        current = torch.cuda.current_stream(self.device)
+        if current.cuda_stream == self.stream.cuda_stream:
+            return torch.empty(shape, dtype=dtype, device=self.device)
+        with self._on_stream():
+            out = torch.empty(shape, dtype=dtype, device=self.device)
+        out.record_stream(current)
+        return out
+
+    def _on_stream(self):
+        cuda = self.torch.cuda
+        return cuda.stream(self.stream if isinstance(self.stream, cuda.Stream) else cuda.ExternalStream(self.stream.cuda_stream, device=self.device))
 
     def close(self):
         h, self._h = getattr(self, "_h", None), None
@@ -198,9 +217,9 @@ class Env:
         n_steps = actions.shape[0] * fs if n_steps is None else int(n_steps)      # every action row is held for frame_skip steps
         assert tuple(actions.shape) == (-(-n_steps // fs), self.n_envs, self.n_actions), tuple(actions.shape)
         if reward is None:
-            reward = torch.empty((n_steps, self.n_envs), dtype=torch.float32, device=self.device)
+            reward = self._empty((n_steps, self.n_envs), torch.float32)
         if done is None:
-            done = torch.empty((n_steps, self.n_envs), dtype=torch.uint8, device=self.device)
+            done = self._empty((n_steps, self.n_envs), torch.uint8)
         fn, name = ((self.lib.k2d_step_static_scratch, "k2d_step_static_scratch") if static_scratch
                     else (self.lib.k2d_step_discrete, "k2d_step_discrete") if discrete else (self.lib.k2d_step, "k2d_step"))
         _check(fn(self._h, actions.data_ptr(), n_steps, reward.data_ptr(), done.data_ptr()), name)
@@ -217,26 +236,24 @@ class Env:
         n_steps = actions.shape[0] * fs if n_steps is None else int(n_steps)
         assert tuple(actions.shape) == (-(-n_steps // fs), self.n_envs, self.n_actions), tuple(actions.shape)
         if reward is None:
-            reward = torch.empty((n_steps, self.n_envs), dtype=torch.float32, device=self.device)
+            reward = self._empty((n_steps, self.n_envs), torch.float32)
         if done is None:
-            done = torch.empty((n_steps, self.n_envs), dtype=torch.uint8, device=self.device)
+            done = self._empty((n_steps, self.n_envs), torch.uint8)
         if obs is None:
-            obs = torch.empty((self.n_envs, self.obs_floats), dtype=torch.float32, device=self.device)
+            obs = self._empty((self.n_envs, self.obs_floats), torch.float32)
         _check(self.lib.k2d_step_obs(self._h, actions.data_ptr(), n_steps, reward.data_ptr(), done.data_ptr(), obs.data_ptr()), "k2d_step_obs")
         return reward, done, obs
 
     def obs(self, out=None):
-        torch = self.torch
         if out is None:
-            out = torch.empty((self.n_envs, self.obs_floats), dtype=torch.float32, device=self.device)
+            out = self._empty((self.n_envs, self.obs_floats), self.torch.float32)
         _check(self.lib.k2d_obs(self._h, out.data_ptr()), "k2d_obs")
         return out
 
     def render(self, out=None):
         """RGBA byte images [n_envs, 125, 125, 4] of the scenes (the pixel observation)"""
-        torch = self.torch
         if out is None:
-            out = torch.empty((self.n_envs, 125, 125, 4), dtype=torch.uint8, device=self.device)
+            out = self._empty((self.n_envs, 125, 125, 4), self.torch.uint8)
         _check(self.lib.k2d_render(self._h, out.data_ptr()), "k2d_render")
         return out
 
@@ -306,9 +323,10 @@ class Env:
         return {name: int(out[i]) for i, name in enumerate(PHASES)}
 
     def enable_trace(self):
-        torch = self.torch
         slots = self.lib.k2d_trace_slots(self._h)
-        self._trace = torch.zeros((self.n_envs, slots, 6), dtype=torch.float32, device=self.device)
+        self._trace = self._empty((self.n_envs, slots, 6), self.torch.float32)
+        with self._on_stream():
+            self._trace.zero_()
         _check(self.lib.k2d_set_trace(self._h, self._trace.data_ptr()), "k2d_set_trace")
         return self._trace
 
