@@ -50,6 +50,7 @@ extern "C" {
 #define K2D_ERR_WAIT (-9)          /* k2d_status: a wait inside k2d_step ran out (see there) */
 #define K2D_ERR_CHECK (-10)        /* k2d_status of a checked build: an index was out of range    */
 #define K2D_ERR_BUILD (-11)        /* the call needs a build of the library with another compile flag */
+#define K2D_ERR_MEMORY (-12)       /* the host ran out of memory                         */
 
 #define K2D_MAX_POLYGONS 12
 #define K2D_MAX_CIRCLES 4

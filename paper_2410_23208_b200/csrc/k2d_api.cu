@@ -4,8 +4,9 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <exception>
+#include <memory>
 #include <mutex>
-#include <new>
 #include <vector>
 
 #include "k2d.h"
@@ -457,6 +458,7 @@ static bool obs_fits(const k2d_state *s) {
 
 #define CUDA_OK(call) do { cudaError_t e_ = (call); if (e_ != cudaSuccess) { std::fprintf(stderr, "k2d: %s failed: %s\n", #call, cudaGetErrorString(e_)); return K2D_ERR_CUDA; } } while (0)
 
+// (The bodies of the entry points that allocate host memory are try blocks: no exception leaves the library.)
 extern "C" {
 
 int k2d_default_config(k2d_config *cfg, int32_t n_envs, int32_t n_polygons, int32_t n_circles, int32_t n_joints, int32_t n_thrusters) {
@@ -502,7 +504,7 @@ int k2d_canonical_words(const k2d_config *cfg) {
     return 6 * N + 2 * slots + 3 * cfg->n_joints + 4;
 }
 
-int k2d_create(const k2d_config *cfg, void *dev_state_buf, void *dev_level_pool_buf, const k2d_level *host_levels, k2d_state **out) {
+int k2d_create(const k2d_config *cfg, void *dev_state_buf, void *dev_level_pool_buf, const k2d_level *host_levels, k2d_state **out) try {
     if (!cfg || !dev_state_buf || !dev_level_pool_buf || !host_levels || !out) return K2D_ERR_NULL;
     *out = nullptr;
     int rc = check_config(cfg);
@@ -510,8 +512,8 @@ int k2d_create(const k2d_config *cfg, void *dev_state_buf, void *dev_level_pool_
     ClassInfo ci;
     if (!pick_class(cfg, &ci)) return K2D_ERR_CONFIG;
     if (((uintptr_t)dev_state_buf & 15) || ((uintptr_t)dev_level_pool_buf & 15)) return K2D_ERR_ALIGN;
-    k2d_state *s = new (std::nothrow) k2d_state();
-    if (!s) return K2D_ERR_ARG;
+    auto owner = std::make_unique<k2d_state>();      // given up on every way out but the last
+    k2d_state *s = owner.get();
     s->cfg = *cfg; s->ci = ci;
     s->G = cfg->lanes_per_scene ? cfg->lanes_per_scene : 16;
     s->stream = (cudaStream_t)cfg->cuda_stream;
@@ -528,7 +530,7 @@ int k2d_create(const k2d_config *cfg, void *dev_state_buf, void *dev_level_pool_
     s->host_levels.assign((size_t)cfg->n_levels * ci.LV_WORDS, 0u);
     for (int l = 0; l < cfg->n_levels; ++l) {
         rc = pack_level(cfg, ci, host_levels + l, s->host_levels.data() + (size_t)l * ci.LV_WORDS);
-        if (rc != K2D_OK) { delete s; return rc; }
+        if (rc != K2D_OK) return rc;
     }
     const BufLayout bl = buffer_layout(cfg, ci);
     s->slots = bl.slots;
@@ -555,11 +557,13 @@ int k2d_create(const k2d_config *cfg, void *dev_state_buf, void *dev_level_pool_
     if (err == cudaSuccess) err = K2D_DISPATCH(setup_step, s, s, num_sms);
     if (err == cudaSuccess) err = cudaMemcpyAsync(s->dev_levels, s->host_levels.data(), s->host_levels.size() * 4, cudaMemcpyHostToDevice, s->stream);
     if (err == cudaSuccess) err = cudaStreamSynchronize(s->stream);
-    if (err != cudaSuccess) { std::fprintf(stderr, "k2d_create: %s\n", cudaGetErrorString(err)); delete s; return K2D_ERR_CUDA; }
+    if (err != cudaSuccess) { std::fprintf(stderr, "k2d_create: %s\n", cudaGetErrorString(err)); return K2D_ERR_CUDA; }
     rc = k2d_reset(s, nullptr);
-    if (rc != K2D_OK) { delete s; return rc; }
-    *out = s;
+    if (rc != K2D_OK) return rc;
+    *out = owner.release();
     return K2D_OK;
+} catch (const std::exception &) {
+    return K2D_ERR_MEMORY;
 }
 
 int k2d_reset(k2d_state *s, const int32_t *host_level_ids) {
@@ -627,7 +631,7 @@ int k2d_render(k2d_state *s, uint8_t *dev_pixels) {
     return K2D_OK;
 }
 
-int k2d_get_state(k2d_state *s, void *host_canonical) {
+int k2d_get_state(k2d_state *s, void *host_canonical) try {
     if (!s || !host_canonical) return K2D_ERR_NULL;
     const k2d_config &c = s->cfg; const ClassInfo &ci = s->ci;
     const int nP = c.n_polygons, nC = c.n_circles, nN = nP + nC, nJ = c.n_joints;
@@ -667,9 +671,11 @@ int k2d_get_state(k2d_state *s, void *host_canonical) {
         for (int k = 0; k < 4; ++k) meta[k] = st[ci.ST_META + k];
     }
     return K2D_OK;
+} catch (const std::exception &) {
+    return K2D_ERR_MEMORY;
 }
 
-int k2d_set_state(k2d_state *s, const void *host_canonical) {
+int k2d_set_state(k2d_state *s, const void *host_canonical) try {
     if (!s || !host_canonical) return K2D_ERR_NULL;
     const k2d_config &c = s->cfg; const ClassInfo &ci = s->ci;
     const int nP = c.n_polygons, nC = c.n_circles, nN = nP + nC, nJ = c.n_joints;
@@ -715,6 +721,8 @@ int k2d_set_state(k2d_state *s, const void *host_canonical) {
     CUDA_OK(cudaStreamSynchronize(s->stream));
     CUDA_OK(cudaMemcpy(s->dev_env, raw.data(), raw.size() * 4, cudaMemcpyHostToDevice));
     return K2D_OK;
+} catch (const std::exception &) {
+    return K2D_ERR_MEMORY;
 }
 
 int k2d_status(k2d_state *s, int64_t *host_counts) {
@@ -732,7 +740,7 @@ int k2d_status(k2d_state *s, int64_t *host_counts) {
     return queue[Q_ERROR] ? K2D_ERR_WAIT : K2D_OK;
 }
 
-int k2d_level_info(const k2d_config *cfg, const k2d_level *host_level, float *host_inv_mass, float *host_inv_inertia, uint8_t *host_collide) {
+int k2d_level_info(const k2d_config *cfg, const k2d_level *host_level, float *host_inv_mass, float *host_inv_inertia, uint8_t *host_collide) try {
     if (!cfg || !host_level) return K2D_ERR_NULL;
     int rc = check_config(cfg);
     if (rc != K2D_OK) return rc;
@@ -754,6 +762,8 @@ int k2d_level_info(const k2d_config *cfg, const k2d_level *host_level, float *ho
                 host_collide[pair_index(nP, nC, a, b)] = (uint8_t)((lv[ci.LV_MASK + internal(a)] >> internal(b)) & 1u);
             }
     return K2D_OK;
+} catch (const std::exception &) {
+    return K2D_ERR_MEMORY;
 }
 
 int k2d_set_trace(k2d_state *s, float *dev_trace) {
@@ -898,6 +908,7 @@ const char *k2d_error_string(int code) {
         case K2D_ERR_LIMIT: return "size beyond a built-in limit";
         case K2D_ERR_CHECK: return "an index check of the checked build failed";
         case K2D_ERR_BUILD: return "this build of the library does not have that feature compiled in";
+        case K2D_ERR_MEMORY: return "the host ran out of memory";
         case K2D_ERR_WAIT: return "a scene group gave up waiting for another; the last step is incomplete";
         default: return "unknown error";
     }

@@ -3,6 +3,8 @@
 import ctypes as C
 import os
 import re
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -83,6 +85,26 @@ def test_create_rejects_bad_arguments_before_touching_the_device():
     broken = packed.copy()
     broken["poly_verts"][0, 1, :, 0] += 0.2
     assert _create(cfg, broken)[0] == -4
+
+
+def test_a_level_pool_too_large_for_the_host_is_an_error_code_not_an_abort():
+    # child process with a limit on its address space; the library packs the pool on the host before it looks at the levels
+    code = """
+import ctypes as C, resource
+import numpy as np
+from paper_2410_23208_b200 import k2d, scenes
+lv = scenes.make_levels("S", 1, 1)
+packed = k2d.pack_levels(lv)
+cfg = k2d.make_config(lv, 1, n_levels=1 << 30)                  # 864 GB of level records
+lib, h = k2d.load_library(), C.c_void_p()
+used = int(open("/proc/self/statm").read().split()[0]) * resource.getpagesize()
+resource.setrlimit(resource.RLIMIT_AS, (used + (1 << 30), resource.RLIM_INFINITY))
+rc = lib.k2d_create(C.byref(cfg), 0x1000, 0x2000, packed.ctypes.data, C.byref(h))
+print(rc, h.value, lib.k2d_error_string(rc).decode())
+"""
+    out = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert out.returncode == 0, out.stderr
+    assert out.stdout.split(maxsplit=2) == ["-12", "None", "the host ran out of memory\n"]
 
 
 def test_error_strings():
