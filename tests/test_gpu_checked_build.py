@@ -60,8 +60,10 @@ def test_no_index_check_fires_on_piles(lanes):
 @pytest.mark.gpu
 def test_no_index_check_fires_through_the_work_queue_and_in_the_batched_solve():
     lv = scenes.make_levels("L", 256, 77, static_prob=0.1)
-    env, ref = _pair(lv, 6200, auto_reset=2, max_episode_steps=10, seed=77, max_fused_steps=24)
-    _run(env, ref, scenes.make_actions(20, 6200, env.n_actions, 77), 20)
+    for n_envs, lanes in ((9600, 8), (6200, 16)):
+        env, ref = _pair(lv, n_envs, auto_reset=2, max_episode_steps=10, seed=77, max_fused_steps=24, lanes_per_scene=lanes)
+        assert env.resident_groups < n_envs
+        _run(env, ref, scenes.make_actions(20, n_envs, env.n_actions, 77), 20)
     lv = scenes.make_levels("M", 64, 78, static_prob=0.1)
     lv["pos"][:16, 1:, 0] *= 0.15
     env, ref = _pair(lv, 64, solver_batch=16)

@@ -32,17 +32,18 @@ def test_benchmark_configuration_matches_the_oracle_on_every_env(lanes, horizon)
     assert d.sum() >= (n_envs * 5 if horizon == 12 else 1)
 
 
-@pytest.mark.parametrize("lanes,n_envs", [(0, 6000), (32, 3000)])
+@pytest.mark.parametrize("lanes,n_envs", [(0, 9600), (16, 6000), (32, 3000)])
 def test_a_few_more_envs_than_resident_groups(lanes, n_envs):
-    # just above the number of scene groups a B200 holds at once (5920 half-warps, 2960 warps for L scenes):
-    # the second chunk of the first envs is handed out while their first chunk may still be running on another
+    # just above the number of scene groups a B200 holds at once (9472 of eight lanes, 5920 of sixteen, 2960 warps for L
+    # scenes): the second chunk of the first envs is handed out while their first chunk may still be running on another
     # group, so groups really wait for one another here
     w = scenes.WORKLOADS[3]
     seed = 77
     lv = scenes.make_levels(w["size"], 256, seed, static_prob=w["static_prob"])
     env, ref = parity.make_pair(lv, n_envs, auto_reset=2, max_episode_steps=10, seed=seed, max_fused_steps=24, lanes_per_scene=lanes)
+    assert 0.9 * n_envs < env.resident_groups < n_envs
     act = scenes.make_actions(40, n_envs, env.n_actions, seed)
-    # launches of 20 steps: work items of 8, 8 and 4 steps
+    # launches of 20 steps: work items of 8, 8 and 4 steps (of 4 with eight lanes)
     (r, d), (rr, dr) = parity.step_both(env, ref, act, chunk=20, n_threads=os.cpu_count() or 1)
     assert np.array_equal(r, rr) and np.array_equal(d, dr)
     err, exact = parity.errors(env, ref)
@@ -185,13 +186,14 @@ def test_discrete_actions_and_the_fused_observation_through_the_sorted_work_queu
     assert exact, err
 
 
-@pytest.mark.parametrize("size,n_envs,lanes", [("L", 7200, 8), ("L", 3200, 32), ("M", 3200, 32)])
+@pytest.mark.parametrize("size,n_envs,lanes", [("L", 7200, 8), ("L", 9600, 8), ("L", 3200, 32), ("M", 3200, 32)])
 def test_one_block_per_sm_form_with_8_and_32_lanes_per_scene(size, n_envs, lanes):
-    # enough envs to fill every scene group of the device at these lane counts, so the step kernel runs as one block per SM
-    # whose warps step in lockstep per scheduler (three warps per scheduler for L scenes at 8 lanes, five otherwise)
+    # the step kernel as one block per SM of the most threads, whose warps step in lockstep per scheduler (four warps per
+    # scheduler at 8 lanes, five at 32): 7200 envs in one wave, the others in more, through the work queue
     index = 3 if size == "L" else 2
     env, ref, seed = _workload_pair(index, n_envs, 24, lanes_per_scene=lanes, auto_reset=2, max_episode_steps=10)
-    assert env.resident_groups <= n_envs and env.items_per_ticket > 32 // lanes      # several warps per ticket: the one-block form
+    assert env.items_per_ticket == (32 // lanes) * (4 if lanes == 8 else 5)      # several warps per ticket: the one-block form
+    assert env.resident_groups == n_envs if n_envs == 7200 else env.resident_groups < n_envs
     act = scenes.make_actions(40, n_envs, env.n_actions, seed)
-    d = _run_and_compare(env, ref, act, 20)               # work items of 8, 8 and 4 steps
+    d = _run_and_compare(env, ref, act, 20)               # through the queue in work items of 8, 8 and 4 steps, or of 4
     assert d.sum() >= 2 * n_envs

@@ -216,9 +216,9 @@ def test_custom_dimensions_and_inactive_entities():
 
 @pytest.mark.parametrize("lanes", [8, 16, 32])
 def test_more_active_pairs_than_lanes_and_than_shared_memory_records(lanes):
-    # every shape of an L scene dropped on the same spot: far more touching pairs than twice the lanes
-    # of a scene, so the step's contacts go through the global-memory scratch; as the pile spreads the
-    # count falls through the range where lanes hold two records each, then one
+    # every shape of an L scene dropped on the same spot: far more touching pairs than a schedule holds (31), so the step's
+    # contacts go through the global-memory scratch as a whole; as the pile spreads the count falls through the range where
+    # only the records beyond the shared-memory ones do
     lv = scenes.make_levels("L", 6, 51)
     rng = np.random.default_rng(51)
     lv["pos"][:, 1:, 0] = rng.uniform(-0.3, 0.3, (6, 15)).astype(np.float32)
@@ -230,7 +230,7 @@ def test_more_active_pairs_than_lanes_and_than_shared_memory_records(lanes):
     (r, d), (rr, dr) = parity.step_both(env, ref, act[:1])
     on = ref.manifold[:, :, 5] > 0                   # 66 polygon pairs own two manifold slots each, the others one
     touching_pairs = (on[:, :132:2] | on[:, 1:132:2]).sum(1) + on[:, 132:].sum(1)
-    assert touching_pairs.max() > lanes + lanes // 2        # more than the records a scene keeps on chip
+    assert touching_pairs.max() > max(31, lanes + lanes // 2)        # more than a schedule holds
     assert np.array_equal(trace.cpu().numpy()[:, :, 5], ref.manifold[:, :, 5])
     err, exact = parity.errors(env, ref)
     assert exact, err
@@ -268,15 +268,16 @@ def test_observation_parity(size):
     assert np.array_equal(got.view(np.uint32), want.view(np.uint32))
 
 
-@pytest.mark.parametrize("size,n_envs,lanes,n_actions", [("S", 40, 0, 0), ("M", 40, 8, 0), ("L", 72, 16, 0), ("L", 24, 32, 16), ("L", 7000, 0, 0)])
+@pytest.mark.parametrize("size,n_envs,lanes,n_actions", [("S", 40, 0, 0), ("M", 40, 8, 0), ("L", 72, 16, 0), ("L", 24, 32, 16), ("L", 7000, 0, 0), ("L", 9600, 0, 0)])
 def test_step_with_observation_in_one_launch(size, n_envs, lanes, n_actions):
     # k2d_step_obs = k2d_step then k2d_obs: one step at a time (the training loop's use), then launches of several steps,
-    # with resets in between; 7000 envs are more than the device holds at once, so those launches are cut into runs and
+    # with resets in between; 9600 envs are more than the device holds at once, so those launches are cut into runs and
     # the observation must come from the last run only
     import torch
     lv = scenes.make_levels(size, min(n_envs, 256), 15, static_prob=0.1, triangle_prob=0.2, fixed_prob=0.2)
     kw = dict(n_actions=n_actions) if n_actions else {}
     env, ref = parity.make_pair(lv, n_envs, auto_reset=2, max_episode_steps=7, seed=9, lanes_per_scene=lanes, max_fused_steps=20, **kw)
+    assert (env.resident_groups < n_envs) == (n_envs == 9600)
     act = scenes.make_actions(3 + 20 + 11, n_envs, env.n_actions, 15)
     for lo, hi in ((0, 1), (1, 2), (2, 3), (3, 23), (23, 34)):
         r, d, o = env.step_obs(torch.from_numpy(act[lo:hi]).cuda())

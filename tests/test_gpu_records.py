@@ -82,6 +82,36 @@ def test_friction_too_large_for_the_fast_limit(lanes):
     _exact(env, ref, scenes.make_actions(40, 24, env.n_actions, 64), chunk=9)
 
 
+@pytest.mark.parametrize("lanes", [8, 16, 32])
+@pytest.mark.parametrize("solver_iters", [1, 8])
+def test_a_normal_impulse_that_overflows_without_friction(lanes, solver_iters):
+    # The friction bound of a frictionless pair is 0 x infinity once its normal impulse overflows.  The value it limits is then no
+    # number either, whichever way the limit is taken; env and oracle agree on every number and on what is none.  (One pair of
+    # movable shapes per scene: what an overflow does to a fixated shape, which the library never writes, is not specified.)
+    dims, levels = scenes.SIZES["M"], []
+    for tilt in (0.0, 0.7, -0.4):
+        nx, ny = -np.sin(tilt), np.cos(tilt)
+        for k, vel in enumerate(((0.0, -3.0e38), (2.0e38, -2.5e38), (-1.0e38, -3.0e38), (0.5, -1.0))):
+            polys = [dict(half=(5.0, 0.5), pos=(-0.5 * nx, -0.5 * ny), angle=tilt, density=2.0, friction=0.0)]
+            box = dict(half=(0.5, 0.5), pos=(0.49 * nx, 0.49 * ny), angle=tilt, vel=vel, density=2.0, friction=0.0)
+            circle = dict(radius=0.8, pos=(0.79 * nx + 2.5 * ny, 0.79 * ny - 2.5 * nx), vel=vel, density=2.0, friction=0.0)
+            levels.append(scenes.custom_level(dims, polygons=polys + [box]))
+            levels.append(scenes.custom_level(dims, polygons=polys, circles=[circle]))
+    env, ref = parity.make_pair(scenes.concat_levels(levels), 24, lanes_per_scene=lanes, solver_iters=solver_iters)
+    act = scenes.make_actions(3, 24, env.n_actions, 68)
+    for k in range(3):
+        (r, d), (rr, dr) = parity.step_both(env, ref, act[k:k + 1])
+        assert np.array_equal(r, rr) and np.array_equal(d, dr)
+        st = env.get_state()
+        for key in parity.STATE_KEYS:
+            assert np.array_equal(st[key], getattr(ref, key), equal_nan=True), key
+        for key in parity.META_KEYS:
+            assert np.array_equal(st[key], getattr(ref, key)), key
+    assert (ref.status[6::8] == 0).all() and (ref.status[7::8] == 0).all() and ref.status.sum() >= 12
+    # a bound that was no number, and a value that was none (with one iteration they stay in the accumulated impulses)
+    assert solver_iters > 1 or (np.isinf(ref.acc[:, :, 0]) & np.isnan(ref.acc[:, :, 1])).sum() >= 12
+
+
 @pytest.mark.parametrize("n_envs", [7103, 7105, 9471, 9472, 9473])
 def test_env_counts_around_the_launch_shapes(n_envs):
     # 48 and 64 scenes per SM on 148 SMs
@@ -95,7 +125,7 @@ def test_env_counts_around_the_launch_shapes(n_envs):
     assert exact, err
 
 
-@pytest.mark.parametrize("size,n_envs,lanes", [("S", 593, 32), ("S", 1183, 32), ("S", 2368, 16), ("M", 2369, 16), ("L", 1185, 32), ("L", 4735, 16), ("S", 4737, 8), ("L", 2663, 0)])
+@pytest.mark.parametrize("size,n_envs,lanes", [("S", 593, 32), ("S", 1183, 32), ("S", 2368, 16), ("M", 2369, 16), ("L", 1185, 32), ("L", 4735, 16), ("S", 4737, 8), ("L", 2663, 0), ("L", 6000, 0)])
 def test_block_sizes_of_launches_of_one_wave(size, n_envs, lanes):
     # one block per SM of 128, 256, 384 or 512 threads, envs on either side of a full device; one step at a time (small blocks
     # where the block would fill an SM) and several
