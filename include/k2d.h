@@ -79,8 +79,7 @@ extern "C" {
  * the batches are solved one after the other; the rows of one batch are all solved against the velocities the batch
  * starts with and applied together afterwards (in canonical order).  The active manifolds are spread over as many batches
  * as possible: the i-th active manifold in canonical order goes to batch i mod n_batches.  While a scene has no more
- * active manifolds than batches this is the sequential solve, bit for bit; the paper's default is B = 16.  The library
- * runs this mode on its general, untuned path (constraint rows in the scratch tail); it is there for fidelity. */
+ * active manifolds than batches this is the sequential solve, bit for bit; the paper's default is B = 16. */
 typedef struct k2d_config {
     int32_t n_envs;                /* >= 1                                                      */
     int32_t n_polygons;            /* 1 .. K2D_MAX_POLYGONS                                     */
@@ -177,7 +176,8 @@ int k2d_reset(k2d_state *s, const int32_t *host_level_ids);
  * floats in {-1, 0, +1}, plus, if dense_kappa is not 0, the paper's auxiliary dense reward
  * kappa * (d_t - d_t+1) with d the distance between the positions of the first green and the
  * first blue shape before and after the step; dev_done [n_steps][n_envs] bytes.  1 <= n_steps <= max_fused_steps.
- * The whole call is one kernel launch; scene state stays on chip between the fused steps. */
+ * The whole call is one launch of the step kernel (with many more envs than the device holds at once, two small launches
+ * that sort them come first, see k2d_step_launches); scene state stays on chip between the fused steps. */
 int k2d_step(k2d_state *s, const float *dev_actions, int32_t n_steps, float *dev_reward, uint8_t *dev_done);
 
 /* The same step with the paper's multi-discrete action space ("Action Space": every motor and
@@ -187,8 +187,8 @@ int k2d_step(k2d_state *s, const float *dev_actions, int32_t n_steps, float *dev
 int k2d_step_discrete(k2d_state *s, const int32_t *dev_actions, int32_t n_steps, float *dev_reward, uint8_t *dev_done);
 
 /* The paper has no counterpart of this call; it exists for one kind of user of this library.
- * k2d_step keeps the contact records of a very crowded scene (far more touching pairs than
- * lanes working on the scene) in the scratch tail of the state buffer, which the caller has to
+ * k2d_step keeps the contact records of a very crowded scene (more touching pairs than it has
+ * room for on chip) in the scratch tail of the state buffer, which the caller has to
  * allocate.  Some callers cannot: a process whose device memory is one arena fixed at start-up,
  * a plug-in handed a pre-sized buffer by its host, code running where cudaMalloc is forbidden
  * (a real-time loop).  For them this variant does exactly what k2d_step does, with the same

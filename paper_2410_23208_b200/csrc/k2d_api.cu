@@ -125,7 +125,7 @@ static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 struct BufLayout { size_t ids_off, chunks_off, env_off, scratch_off, total; int slots; };
 static BufLayout buffer_layout(const k2d_config *cfg, const ClassInfo &ci) {
     BufLayout b{};
-    // every scene group of a launch can end up stepping an env, so the scratch covers whole blocks (up to 16 groups each)
+    // a slot per env in a launch of one wave, a slot per scene group in others; setup_step keeps the launch within them
     const size_t slots = ((cfg->n_envs < kMaxSlots ? cfg->n_envs : kMaxSlots) + 15) / 16 * 16;
     // the sequential contact solve needs less per scene group, so the same memory serves more groups
     b.slots = cfg->solver_batch > 0 ? (int)slots : (int)(slots * ci.SCRATCH_WORDS_BATCHED / ci.SCRATCH_WORDS);
@@ -410,8 +410,8 @@ static StepParams step_params(const k2d_state *s, const float *dev_actions, int 
     return prm;
 }
 
-// Launches of at least kOrderMinSteps steps with two or more scenes per warp and more envs than the device holds scene groups
-// first sort the envs by what their steps cost (see k2d_order_count_kernel); the order lives in the words through which k2d_reset
+// Launches with more envs than the device holds scene groups (how many more: uses_order) first sort the envs by what their steps
+// cost (see k2d_order_count_kernel), those of fewer than kOrderMinSteps steps only now and then (reuses_order); the order lives in the words through which k2d_reset
 // hands over level ids, and k2d_reset leaves them as the order by index: a launch recorded into a graph while it reused an
 // order finds a permutation there whatever was called since.
 constexpr int kOrderMinSteps = 8, kOrderShortLaunches = 16;
