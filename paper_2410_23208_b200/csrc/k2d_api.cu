@@ -297,7 +297,10 @@ static cudaError_t launch_after(void (*kernel)(P...), int grid, int threads, siz
 // 33.8 / 31.5, M x 4096 31.5 / 28.4 and 37.3 / 34.6, L x 2048 31.8 / 31.5 and 39.9 / 38.1; with smaller blocks it depends (L x 3000
 // 37.5 / 41.2), with two steps the lockstep is worth more (L x 4096 74.6 / 77.3).
 constexpr int kApartThreads = 512;
-// calls f with the step kernel in blocks of block_threads threads (a multiple of kSmallBlock up to THREADS)
+// calls f with the step kernel in blocks of block_threads threads (a multiple of kSmallBlock up to THREADS).  All multiples are
+// compiled: without the one between 256 and 512 threads the envs that need it run in 512, where some of an SM's four groups of warps
+// get no envs and the others get more (32 steps, 384 / 512 threads: S x 5003 649 / 718 us, M x 3500 614 / 656, M x 5003 794 / 860,
+// L x 1700 786 / 848, L x 3500 988 / 1090, L x 6000 1211 / 1351).
 template <class SC, int G, int THREADS, class F>
 static cudaError_t with_step_kernel(int block_threads, F f) {
     if constexpr (THREADS > kSmallBlock) {

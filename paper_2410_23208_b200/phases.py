@@ -1,7 +1,7 @@
 """Where a step's time goes: runs a benchmark workload on the build of the library whose step kernel counts SM cycles
 per phase (-DK2D_PHASE_CLOCKS) and prints each phase's share.
 
-    python -m paper_2410_23208_b200.phases [--workload 3] [--envs N] [--launches 4] [--fused 32]
+    python -m paper_2410_23208_b200.phases [--workload 3] [--envs N] [--launches 4] [--fused 32] [--solver-batch B]
 
 The counting build is slower than the library proper (two clock reads and an atomic add per phase boundary), so the shares
 are what to read, not the rate.
@@ -14,14 +14,14 @@ import json
 from . import k2d, scenes
 
 
-def phase_shares(workload: int = 3, n_envs: int = 0, launches: int = 4, fused: int = 32, lanes: int = 0) -> dict:
+def phase_shares(workload: int = 3, n_envs: int = 0, launches: int = 4, fused: int = 32, lanes: int = 0, solver_batch: int = 0) -> dict:
     import torch
     w = scenes.WORKLOADS[workload]
     n_envs = n_envs or w["n_envs"]
     seed = scenes.workload_seed(workload)
     levels = scenes.make_levels(w["size"], w["n_levels"], seed, static_prob=w["static_prob"])
     env = k2d.Env(levels, n_envs, phase_clocks=True, auto_reset=w["auto_reset"], max_episode_steps=w["max_episode_steps"], seed=seed,
-                  max_fused_steps=fused, lanes_per_scene=lanes)
+                  max_fused_steps=fused, lanes_per_scene=lanes, solver_batch=solver_batch)
     actions = torch.from_numpy(scenes.make_actions(fused, n_envs, env.n_actions, seed)).cuda()
     env.step(actions)                       # warm-up launch, not counted
     env.phase_cycles()
@@ -43,9 +43,10 @@ def main():
     ap.add_argument("--launches", type=int, default=4)
     ap.add_argument("--fused", type=int, default=32)
     ap.add_argument("--lanes", type=int, default=0)
+    ap.add_argument("--solver-batch", type=int, default=0, help="the batched contact solve: its rounds are worked out in the phase \"levels\"")
     ap.add_argument("--json", action="store_true")
     args = ap.parse_args()
-    out = phase_shares(args.workload, args.envs, args.launches, args.fused, args.lanes)
+    out = phase_shares(args.workload, args.envs, args.launches, args.fused, args.lanes, args.solver_batch)
     if args.json:
         print(json.dumps(out))
         return
