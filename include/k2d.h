@@ -300,6 +300,10 @@ int k2d_set_wait_limit(k2d_state *s, uint32_t polls);
  * uses these instead of libm so that results are reproducible bit for bit). */
 int k2d_eval_sincos_tanh(const float *dev_x, int32_t n, float *dev_cos, float *dev_sin, float *dev_tanh, void *cuda_stream);
 
+/* Test aid: the kernels' branch-free reciprocal and square root of dev_b and quotient dev_a / dev_b.  Correctly rounded for
+ * 2^-60 <= |b| < 2^60 and a of the same range or +0 (roots: b > 0); outside of it the kernels use the ordinary operations. */
+int k2d_eval_quotients(const float *dev_a, const float *dev_b, int32_t n, float *dev_reciprocal, float *dev_quotient, float *dev_root, void *cuda_stream);
+
 /* Measurement aid, not part of the step: runs chains of dependent fused multiply-adds on every SM of the device (eight
  * independent chains per thread, 2048 threads per SM) on the default stream and returns the FP32 rate they reach, in
  * TFLOP/s (a multiply-add counts 2), in *host_tflops: the measured counterpart of SMs x 128 lanes x 2 x clock.

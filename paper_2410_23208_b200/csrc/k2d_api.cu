@@ -826,6 +826,14 @@ int k2d_eval_sincos_tanh(const float *dev_x, int32_t n, float *dev_cos, float *d
     return K2D_OK;
 }
 
+int k2d_eval_quotients(const float *dev_a, const float *dev_b, int32_t n, float *dev_reciprocal, float *dev_quotient, float *dev_root, void *cuda_stream) {
+    if (!dev_a || !dev_b) return K2D_ERR_NULL;
+    if (n < 1) return K2D_ERR_ARG;
+    k2d_eval_quotients_kernel<<<(n + 255) / 256, 256, 0, (cudaStream_t)cuda_stream>>>(dev_a, dev_b, n, dev_reciprocal, dev_quotient, dev_root);
+    CUDA_OK(cudaGetLastError());
+    return K2D_OK;
+}
+
 // ---- k2d_step for callers that cannot provide the overflow scratch: it lives in the library image.
 // One array per device that loads the library, held until the process exits.
 static __device__ __align__(256) uint32_t k2d_static_scratch[(size_t)K2D_STATIC_SCRATCH_MAX_ENVS * ClassL::SCRATCH_WORDS_BATCHED];

@@ -20,7 +20,7 @@ EXPORTS = (
     "k2d_default_config", "k2d_state_bytes", "k2d_state_bytes_no_scratch", "k2d_level_pool_bytes", "k2d_create", "k2d_reset", "k2d_step",
     "k2d_step_discrete", "k2d_step_static_scratch", "k2d_step_obs", "k2d_obs", "k2d_render",
     "k2d_obs_floats", "k2d_canonical_words", "k2d_get_state", "k2d_set_state", "k2d_status", "k2d_level_info",
-    "k2d_set_trace", "k2d_trace_slots", "k2d_is_checked_build", "k2d_phase_cycles", "k2d_resident_groups", "k2d_lanes_per_scene", "k2d_step_launches", "k2d_items_per_ticket", "k2d_set_wait_limit", "k2d_eval_sincos_tanh", "k2d_measure_fp32_peak", "k2d_error_string", "k2d_destroy",
+    "k2d_set_trace", "k2d_trace_slots", "k2d_is_checked_build", "k2d_phase_cycles", "k2d_resident_groups", "k2d_lanes_per_scene", "k2d_step_launches", "k2d_items_per_ticket", "k2d_set_wait_limit", "k2d_eval_sincos_tanh", "k2d_eval_quotients", "k2d_measure_fp32_peak", "k2d_error_string", "k2d_destroy",
 )
 
 
@@ -96,6 +96,7 @@ def load_library(checked: bool = False, phase_clocks: bool = False):
         lib.k2d_step_launches.argtypes = [vp, i32]
         lib.k2d_items_per_ticket.argtypes = [vp]
         lib.k2d_eval_sincos_tanh.argtypes = [vp, i32, vp, vp, vp, vp]
+        lib.k2d_eval_quotients.argtypes = [vp, vp, i32, vp, vp, vp, vp]
         lib.k2d_measure_fp32_peak.argtypes = [i32, vp, C.c_size_t, vp]
         lib.k2d_error_string.argtypes = [C.c_int]
         lib.k2d_error_string.restype = C.c_char_p
@@ -351,6 +352,18 @@ def eval_sincos_tanh(x):
     _check(lib.k2d_eval_sincos_tanh(x.data_ptr(), x.numel(), c.data_ptr(), s.data_ptr(), t.data_ptr(),
                                     torch.cuda.current_stream(x.device).cuda_stream), "k2d_eval_sincos_tanh")
     return c, s, t
+
+
+def eval_quotients(a, b):
+    """The kernels' branch-free 1 / b, a / b and sqrt(b) of CUDA float32 tensors (see k2d_eval_quotients)."""
+    import torch
+    lib = load_library()
+    a, b = a.contiguous(), b.contiguous()
+    assert a.shape == b.shape and a.dtype == b.dtype == torch.float32
+    r, q, s = torch.empty_like(b), torch.empty_like(b), torch.empty_like(b)
+    _check(lib.k2d_eval_quotients(a.data_ptr(), b.data_ptr(), b.numel(), r.data_ptr(), q.data_ptr(), s.data_ptr(),
+                                  torch.cuda.current_stream(b.device).cuda_stream), "k2d_eval_quotients")
+    return r, q, s
 
 
 def measure_fp32_peak(device: int = 0) -> float:

@@ -31,6 +31,52 @@ def test_sincos_tanh_bit_equal_to_the_oracle():
         assert np.array_equal(got.cpu().numpy().view(np.uint32), want.view(np.uint32))
 
 
+def test_quotients_and_roots_of_moderate_numbers():
+    """every positive float32 of [2^-60, 2^60): the reciprocal and the root are the correctly rounded ones (IEEE operations of
+    numpy for two binades, of torch for the rest), and so are quotients by each of them, signs and a zero numerator included"""
+    import torch
+    gen = torch.Generator("cuda").manual_seed(1)
+    for exponent in range(67, 187, 4):
+        bits = torch.arange(exponent << 23, min(exponent + 4, 187) << 23, dtype=torch.int32, device="cuda")
+        b = bits.view(torch.float32)
+        a_bits = torch.randint(67 << 23, 187 << 23, bits.shape, dtype=torch.int32, device="cuda", generator=gen)
+        a = torch.where(bits % 97 == 0, 0.0, a_bits.view(torch.float32))
+        a = torch.where((bits % 2 == 0) & (a != 0), -a, a)
+        r, q, s = k2d.eval_quotients(a, b)
+        for got, want in ((r, 1.0 / b), (q, a / b), (s, torch.sqrt(b))):
+            assert torch.equal(got.view(torch.int32), want.view(torch.int32)), exponent
+        if exponent == 127:
+            n = 2 << 23
+            an, bn = a[:n].cpu().numpy(), b[:n].cpu().numpy()
+            for got, want in ((r, np.float32(1.0) / bn), (q, an / bn), (s, np.sqrt(bn))):
+                assert np.array_equal(got[:n].cpu().numpy().view(np.uint32), want.view(np.uint32))
+        r, q, _ = k2d.eval_quotients(-a, -b)
+        assert torch.equal(r, -(1.0 / b)) and torch.equal(q[a != 0], (a / b)[a != 0])
+
+
+@pytest.mark.parametrize("size,lanes", [("S", 32), ("M", 16), ("L", 8)])
+@pytest.mark.parametrize("density", [1e-21, 1.0, 3e18])
+def test_masses_beyond_the_branch_free_quotients(size, lanes, density):
+    """inverse masses on both sides of 2^60 (and the ordinary ones), frictionless shapes, no positional corrections: the records
+    whose operands the branch-free operations do not take go through the ordinary ones, with the oracle's bits"""
+    n_envs = 24
+    lv = scenes.make_levels(size, n_envs, 1013, static_prob=0.1)
+    lv["density"] = (lv["density"] * np.float32(density)).astype(np.float32)
+    lv["motor_power"] = (lv["motor_power"] * np.float32(density)).astype(np.float32)
+    lv["thr_power"] = (lv["thr_power"] * np.float32(density)).astype(np.float32)
+    lv["friction"][::3] = 0.0
+    if density > 1.0:
+        lv["joint_active"][:] = 0                  # the determinant of a joint's matrix is the square of such a small number
+    else:
+        lv["density"][1::4, -2:] = 1.0             # scenes with both kinds of masses
+    for kw in ({}, dict(contact_beta=0.0, joint_beta=0.0)):
+        env, ref = parity.make_pair(lv, n_envs, lanes_per_scene=lanes, max_fused_steps=64, **kw)
+        act = scenes.make_actions(60, n_envs, env.n_actions, 13)
+        (r, d), (rr, dr) = parity.step_both(env, ref, act)
+        assert np.array_equal(r, rr) and np.array_equal(d, dr)
+        assert np.isfinite(ref.pos).all() and parity.errors(env, ref)[1]
+
+
 @pytest.mark.parametrize("size,n_envs,seed", [("S", 16, 1000), ("M", 48, 1002), ("L", 80, 1003)])
 def test_step_parity_1_16_and_100_steps(size, n_envs, seed):
     lv = scenes.make_levels(size, n_envs, seed, static_prob=0.1)
