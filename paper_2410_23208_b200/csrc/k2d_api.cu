@@ -189,6 +189,9 @@ static int pack_level(const k2d_config *cfg, const ClassInfo &ci, const k2d_leve
                 w[ci.LV_ELEN + 4 * q + k] = f2u((float)len);
                 ext = std::fmax(ext, std::fmax(std::fabs(x0), std::fabs(y0)));
             }
+            // a triangle's fourth vertex, normal and edge are its first: loops over four of them need no count
+            if (nv == 3)
+                for (int f : { ci.LV_PVX, ci.LV_PVY, ci.LV_PNX, ci.LV_PNY, ci.LV_ELEN }) w[f + 4 * q + 3] = w[f + 4 * q];
             if (!(area2 > 0.0)) return K2D_ERR_LEVEL;
             if (std::hypot(cxs / (3.0 * area2), cys / (3.0 * area2)) > 1e-3 * ext) return K2D_ERR_LEVEL;  // centroid at the origin
             const double rho = L->density[i];

@@ -77,6 +77,31 @@ def test_masses_beyond_the_branch_free_quotients(size, lanes, density):
         assert np.isfinite(ref.pos).all() and parity.errors(env, ref)[1]
 
 
+@pytest.mark.parametrize("lanes", [8, 16, 32])
+@pytest.mark.parametrize("size", ["S", "M", "L"])
+def test_separating_axes_of_polygons_no_minimum_orders(size, lanes):
+    """shapes so far out that products of coordinates could overflow, and angles beyond the sine's range (their vertices are no
+    numbers), between ordinary scenes of the same warps, with triangles: every env that stays finite has the oracle's bits"""
+    n_envs = 40
+    lv = scenes.make_levels(size, n_envs, 1014, static_prob=0.2, triangle_prob=0.5)
+    lv["joint_active"][:] = 0
+    lv["thr_active"][:] = 0
+    lv["angle"][1::5, 2] = 2.0e6
+    lv["angle"][2::5, 1:4] = -3.0e6
+    lv["pos"][3::5, 2] = 3.0e18
+    lv["pos"][3::5, 3] = lv["pos"][3::5, 2]
+    lv["pos"][4::10, 1:3] = -2.0e25
+    env, ref = parity.make_pair(lv, n_envs, lanes_per_scene=lanes, max_fused_steps=32)
+    act = np.zeros((20, n_envs, env.n_actions), np.float32)
+    (r, d), (rr, dr) = parity.step_both(env, ref, act)
+    ok = ref.status == 0
+    assert ok.mean() > 0.5 and np.array_equal(d[:, ok], dr[:, ok]) and np.array_equal(r[:, ok], rr[:, ok])
+    st = env.get_state()
+    assert np.array_equal(st["status"], ref.status)
+    for k in ("pos", "angle", "vel", "angvel", "acc"):
+        assert np.array_equal(st[k][ok].view(np.uint32), np.ascontiguousarray(getattr(ref, k)[ok]).view(np.uint32)), k
+
+
 @pytest.mark.parametrize("size,n_envs,seed", [("S", 16, 1000), ("M", 48, 1002), ("L", 80, 1003)])
 def test_step_parity_1_16_and_100_steps(size, n_envs, seed):
     lv = scenes.make_levels(size, n_envs, seed, static_prob=0.1)
