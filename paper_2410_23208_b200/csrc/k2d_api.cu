@@ -309,14 +309,15 @@ static cudaError_t with_step_kernel(int block_threads, F f) {
     if constexpr (THREADS > kSmallBlock) {
         if (block_threads < THREADS) return with_step_kernel<SC, G, THREADS - kSmallBlock>(block_threads, f);
     }
-    return f(k2d_step_kernel<SC, G, THREADS>);
+    return f(k2d_step_kernel<SC, G, THREADS, 1>);
 }
 template <class SC, int G>
 static cudaError_t launch_step(const k2d_state *s, const StepParams &prm) {
     const bool apart = prm.n_steps == 1 && s->apart_grid > 0;
-    const int grid = apart ? s->apart_grid : s->grid, threads = apart ? kSmallBlock : s->block_threads;
-    return with_step_kernel<SC, G, step_block_threads<SC, G>()>(threads, [&](auto *kernel) {
-        return launch_after(kernel, grid, threads, apart ? step_block_smem<SC, G>(kSmallBlock) : s->smem_bytes, s->stream, prm);
+    if (apart)
+        return launch_after(k2d_step_kernel<SC, G, kSmallBlock, kSmallBlocksPerSM>, s->apart_grid, kSmallBlock, step_block_smem<SC, G>(kSmallBlock), s->stream, prm);
+    return with_step_kernel<SC, G, step_block_threads<SC, G>()>(s->block_threads, [&](auto *kernel) {
+        return launch_after(kernel, s->grid, s->block_threads, s->smem_bytes, s->stream, prm);
     });
 }
 // Launch shape of the step kernel for this handle: one block per SM, of the fewest threads that give every env a scene group (one
@@ -351,8 +352,9 @@ static cudaError_t setup_step(k2d_state *s, int num_sms) {
     if (threads >= kApartThreads && grid * GPB >= n) {
         int small_per_sm = 0;
         const size_t smem = step_block_smem<SC, G>(kSmallBlock);
-        err = cudaFuncSetAttribute(k2d_step_kernel<SC, G, kSmallBlock>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (err == cudaSuccess) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&small_per_sm, k2d_step_kernel<SC, G, kSmallBlock>, kSmallBlock, smem);
+        auto *kernel = k2d_step_kernel<SC, G, kSmallBlock, kSmallBlocksPerSM>;
+        err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (err == cudaSuccess) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&small_per_sm, kernel, kSmallBlock, smem);
         if (err != cudaSuccess) return err;
         const int need = (n + kSmallBlock / G - 1) / (kSmallBlock / G);
         if (need <= num_sms * small_per_sm) s->apart_grid = need;
