@@ -148,3 +148,17 @@ def test_state_of_scenes_without_joints():
     _exact(env, ref, scenes.make_actions(5, 8, env.n_actions, 67))
     env.set_state(env.get_state())
     _exact(env, ref, scenes.make_actions(5, 8, env.n_actions, 68))
+
+
+@pytest.mark.parametrize("size,n_envs,lanes", [("S", 1, 32), ("S", 129, 16), ("M", 37, 16), ("L", 130, 8), ("L", 600, 0), ("S", 5003, 0), ("S", 20011, 0)])
+def test_work_counters_of_blocks_of_every_fill(size, n_envs, lanes):
+    """counts that leave the blocks together: one scene, blocks partly filled, several blocks, small blocks beside one another
+    (one step of many envs), several waves; and launches long enough for the groups to write theirs out on the way"""
+    lv = scenes.make_levels(size, min(n_envs, 64), 67, static_prob=0.1)
+    env, ref = parity.make_pair(lv, n_envs, broadphase=1, lanes_per_scene=lanes, auto_reset=2, max_episode_steps=40, seed=67, max_fused_steps=300)
+    for i, n_steps in enumerate([1, 1, 2] + ([300] if n_envs < 200 else [9])):
+        act = scenes.make_actions(n_steps, n_envs, env.n_actions, 670 + i)
+        (r, d), (rr, dr) = parity.step_both(env, ref, act, n_threads=8)
+        assert np.array_equal(r, rr) and np.array_equal(d, dr)
+        assert parity.counters_match(env, ref), (n_steps, env.status(), ref.counters)
+    assert parity.errors(env, ref)[1]
