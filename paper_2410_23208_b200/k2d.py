@@ -391,18 +391,34 @@ def noop_outcomes(levels: dict, n_steps: int, device: int = 0, chunk: int = 32, 
     auto-reset; returns +1 / -1 / 0 per level (see first_outcomes).  The paper's level generator rejects levels
     that the no-op policy solves ("trivially solvable"); this is that rollout, run by the CUDA library."""
     import torch
+    if n_steps < 1:
+        raise ValueError("n_steps must be at least 1")
     n = levels["pos"].shape[0]
     env = Env(levels, n, device=device, auto_reset=RESET_NONE, max_fused_steps=chunk, **cfg_kw)
     zeros = torch.zeros((chunk, n, env.n_actions), dtype=torch.float32, device=env.device)
-    # all launches are enqueued before the host waits for the first result
+    # All launches are enqueued before the host waits for the first result; a launch's results are fetched, and searched for first
+    # done steps, while later ones run (1024 L levels, 256 steps: 7.19 ms, fetched and searched at the end 7.59 ms).
     reward = torch.empty((n_steps, n), dtype=torch.float32, device=env.device)
     done = torch.empty((n_steps, n), dtype=torch.uint8, device=env.device)
+    parts = []
     for s0 in range(0, n_steps, chunk):
-        k = min(chunk, n_steps - s0)
-        env.step(zeros[:k], reward[s0:s0 + k], done[s0:s0 + k])
-    r, d = reward.cpu().numpy(), done.cpu().numpy()
+        part = slice(s0, min(s0 + chunk, n_steps))
+        env.step(zeros[:part.stop - s0], reward[part], done[part])
+        with env._on_stream():
+            stepped = torch.cuda.Event()
+            stepped.record()
+        parts.append((part, stepped))
+    fetch = torch.cuda.Stream(env.device)
+    out, is_open = np.zeros(n, np.int8), np.ones(n, bool)
+    with torch.cuda.stream(fetch):
+        for part, stepped in parts:
+            fetch.wait_event(stepped)
+            r, d = reward[part].cpu().numpy(), done[part].cpu().numpy()
+            ends = is_open & d.any(axis=0)
+            out[ends] = first_outcomes(r, d)[ends]
+            is_open &= ~ends
     env.close()
-    return first_outcomes(r, d)
+    return out
 
 
 def shard_envs(n_envs_total: int, rank: int, world_size: int):
