@@ -817,6 +817,25 @@ int k2d_phase_cycles(k2d_state *s, uint64_t *host_cycles, int32_t n) {
 #endif
 }
 
+int k2d_slow_paths(k2d_state *s, uint64_t *host_counts, int32_t n) {
+    if (!s || !host_counts) return K2D_ERR_NULL;
+    if (n < 0 || n > K2D_SLOW_PATHS) return K2D_ERR_ARG;
+    static_assert(K2D_SLOW_PATHS == SLOW_COUNT, "the header's count is the kernels'");
+#ifdef K2D_PHASE_CLOCKS
+    CUDA_OK(cudaSetDevice(s->cfg.device));
+    CUDA_OK(cudaStreamSynchronize(s->stream));
+    unsigned long long sums[SLOW_COUNT];
+    CUDA_OK(cudaMemcpyFromSymbol(sums, k2d_slow_sums, sizeof(sums)));
+    for (int i = 0; i < n; ++i) host_counts[i] = (uint64_t)sums[i];
+    std::memset(sums, 0, sizeof(sums));
+    CUDA_OK(cudaMemcpyToSymbol(k2d_slow_sums, sums, sizeof(sums)));
+    return K2D_OK;
+#else
+    for (int i = 0; i < n; ++i) host_counts[i] = 0;
+    return K2D_ERR_BUILD;
+#endif
+}
+
 int k2d_set_wait_limit(k2d_state *s, uint32_t polls) {
     if (!s) return K2D_ERR_NULL;
     s->wait_limit = polls < 64u ? 64u : polls;

@@ -20,7 +20,7 @@ EXPORTS = (
     "k2d_default_config", "k2d_state_bytes", "k2d_state_bytes_no_scratch", "k2d_level_pool_bytes", "k2d_create", "k2d_reset", "k2d_step",
     "k2d_step_discrete", "k2d_step_static_scratch", "k2d_step_obs", "k2d_obs", "k2d_render",
     "k2d_obs_floats", "k2d_canonical_words", "k2d_get_state", "k2d_set_state", "k2d_status", "k2d_level_info",
-    "k2d_set_trace", "k2d_trace_slots", "k2d_is_checked_build", "k2d_phase_cycles", "k2d_resident_groups", "k2d_lanes_per_scene", "k2d_step_launches", "k2d_items_per_ticket", "k2d_set_wait_limit", "k2d_eval_sincos_tanh", "k2d_eval_quotients", "k2d_measure_fp32_peak", "k2d_error_string", "k2d_destroy",
+    "k2d_set_trace", "k2d_trace_slots", "k2d_is_checked_build", "k2d_phase_cycles", "k2d_slow_paths", "k2d_resident_groups", "k2d_lanes_per_scene", "k2d_step_launches", "k2d_items_per_ticket", "k2d_set_wait_limit", "k2d_eval_sincos_tanh", "k2d_eval_quotients", "k2d_measure_fp32_peak", "k2d_error_string", "k2d_destroy",
 )
 
 
@@ -57,6 +57,7 @@ _libs = {}
 
 PHASES = ("geometry", "actuators", "joint_prestep", "box_test", "narrowphase", "records", "levels", "warm_start", "iterations",
           "integrate_correct", "epilogue", "memory_record_solve", "load", "store")
+SLOW_PATHS = ("axes",)
 
 
 def load_library(checked: bool = False, phase_clocks: bool = False):
@@ -91,6 +92,7 @@ def load_library(checked: bool = False, phase_clocks: bool = False):
         lib.k2d_trace_slots.argtypes = [vp]
         lib.k2d_set_wait_limit.argtypes = [vp, C.c_uint32]
         lib.k2d_phase_cycles.argtypes = [vp, vp, i32]
+        lib.k2d_slow_paths.argtypes = [vp, vp, i32]
         lib.k2d_resident_groups.argtypes = [vp]
         lib.k2d_lanes_per_scene.argtypes = [vp]
         lib.k2d_step_launches.argtypes = [vp, i32]
@@ -322,6 +324,13 @@ class Env:
         out = (C.c_uint64 * len(PHASES))()
         _check(self.lib.k2d_phase_cycles(self._h, out, len(PHASES)), "k2d_phase_cycles")
         return {name: int(out[i]) for i, name in enumerate(PHASES)}
+
+    def slow_paths(self) -> dict:
+        """measurement aid (phase_clocks=True builds): how often the step kernel took code that is right for any operand, but slow,
+        since the last call (see k2d_slow_paths); clears the counts"""
+        out = (C.c_uint64 * len(SLOW_PATHS))()
+        _check(self.lib.k2d_slow_paths(self._h, out, len(SLOW_PATHS)), "k2d_slow_paths")
+        return {name: int(out[i]) for i, name in enumerate(SLOW_PATHS)}
 
     def enable_trace(self):
         slots = self.lib.k2d_trace_slots(self._h)

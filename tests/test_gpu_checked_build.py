@@ -173,3 +173,39 @@ def test_phase_clocks_count_every_phase_and_change_no_result():
     plain = k2d.Env(lv, 8)
     with pytest.raises(k2d.K2DError, match="build"):
         plain.phase_cycles()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("size,lanes", [("S", 16), ("M", 8), ("L", 8), ("L", 16)])
+def test_frozen_scenes_do_not_send_their_neighbours_through_the_compared_axes(size, lanes):
+    """a scene that is frozen (its words are no numbers) and the empty groups of a last, partly filled warp leave the path of the
+    other scenes of a warp alone; a scene that is stepped at such coordinates does not"""
+    import torch
+    n_envs = 41
+    lv = scenes.make_levels(size, n_envs, 78, static_prob=0.1)
+    env, other = (k2d.Env(lv, n_envs, phase_clocks=True, lanes_per_scene=lanes) for _ in range(2))
+    act = torch.from_numpy(scenes.make_actions(12, n_envs, env.n_actions, 78)).cuda()
+    frozen = np.arange(n_envs) % 4 == 1
+    st = env.get_state()
+    st["pos"][frozen] = np.nan
+    st["status"][frozen] = 1
+    env.set_state(st)
+    env.slow_paths()
+    reward, done = env.step(act)
+    assert env.slow_paths()["axes"] == 0
+    want_r, want_d = other.step(act)
+    keep = torch.from_numpy(~frozen).cuda()
+    assert torch.equal(reward[:, keep], want_r[:, keep]) and torch.equal(done[:, keep], want_d[:, keep])
+    assert bool((done[:, ~keep] == 1).all()) and bool((reward[:, ~keep] == 0).all())
+    got, want = env.get_state(), other.get_state()
+    for k in parity.STATE_KEYS:
+        assert np.array_equal(got[k][~frozen].view(np.uint32), want[k][~frozen].view(np.uint32)), k
+    st = other.get_state()
+    st["pos"][7, 1] = 3.0e18
+    other.set_state(st)
+    other.slow_paths()
+    other.step(act)
+    assert 0 < other.slow_paths()["axes"] <= 12 and other.slow_paths()["axes"] == 0      # one warp of the launch; reading clears
+    plain = k2d.Env(lv, 8)
+    with pytest.raises(k2d.K2DError, match="build"):
+        plain.slow_paths()
