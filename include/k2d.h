@@ -292,9 +292,10 @@ int k2d_phase_cycles(k2d_state *s, uint64_t *host_cycles, int32_t n);
 
 /* Measurement aid of the same build: how often the step kernel took code that is right for any operand, but slow, since the last
  * call; waits for the handle's stream, copies the first n (<= K2D_SLOW_PATHS) counts and clears them.  In order: steps of a warp
- * that compared polygon vertices one by one (some coordinate of a scene it steps beyond 2^60, or no number).  In any other
- * build: zeros and K2D_ERR_BUILD. */
-#define K2D_SLOW_PATHS 1
+ * that compared polygon vertices one by one (some coordinate of a scene it steps beyond 2^60, or no number);
+ * joint rows, and contact records, with an operand of a quotient or root outside 2^-60 .. 2^60 that is not 0.  In any other build:
+ * zeros and K2D_ERR_BUILD. */
+#define K2D_SLOW_PATHS 3
 int k2d_slow_paths(k2d_state *s, uint64_t *host_counts, int32_t n);
 
 /* Test aid.  With more envs than the device holds scene groups, k2d_step hands out runs of 8 (or 4) steps of an env to whichever

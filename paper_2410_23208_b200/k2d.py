@@ -57,7 +57,7 @@ _libs = {}
 
 PHASES = ("geometry", "actuators", "joint_prestep", "box_test", "narrowphase", "records", "levels", "warm_start", "iterations",
           "integrate_correct", "epilogue", "memory_record_solve", "load", "store")
-SLOW_PATHS = ("axes",)
+SLOW_PATHS = ("axes", "joint_rows", "records")
 
 
 def load_library(checked: bool = False, phase_clocks: bool = False):

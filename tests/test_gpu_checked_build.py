@@ -209,3 +209,26 @@ def test_frozen_scenes_do_not_send_their_neighbours_through_the_compared_axes(si
     plain = k2d.Env(lv, 8)
     with pytest.raises(k2d.K2DError, match="build"):
         plain.slow_paths()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("size,lanes", [("S", 32), ("M", 8), ("L", 8), ("L", 16)])
+def test_constants_of_zero_are_ordinary_operands(size, lanes):
+    """with the positional corrections switched off and no friction, joint rows and contact records take the branch-free quotients
+    and roots as ever; masses beyond their range do not"""
+    n_envs = 40
+    lv = scenes.make_levels(size, n_envs, 79, static_prob=0.1)
+    lv["friction"][:] = 0.0
+    env, ref = parity.make_pair(lv, n_envs, phase_clocks=True, lanes_per_scene=lanes, joint_beta=0.0, contact_beta=0.0, joint_alpha=0.0, slop=0.0)
+    act = scenes.make_actions(30, n_envs, env.n_actions, 79)
+    env.slow_paths()
+    (r, d), (rr, dr) = parity.step_both(env, ref, act)
+    assert env.slow_paths() == {"axes": 0, "joint_rows": 0, "records": 0}
+    assert np.array_equal(r, rr) and np.array_equal(d, dr) and ref.counters[2] > 0 and parity.errors(env, ref)[1]
+    for k in ("density", "motor_power", "thr_power"):
+        lv[k][:] *= np.float32(1e-21)
+    env, ref = parity.make_pair(lv, n_envs, phase_clocks=True, lanes_per_scene=lanes)
+    env.slow_paths()
+    (r, d), (rr, dr) = parity.step_both(env, ref, np.zeros_like(act))
+    slow = env.slow_paths()
+    assert slow["joint_rows"] > 0 and slow["records"] > 0 and parity.errors(env, ref)[1]
