@@ -33,7 +33,8 @@ def test_sincos_tanh_bit_equal_to_the_oracle():
 
 def test_quotients_and_roots_of_moderate_numbers():
     """every positive float32 of [2^-60, 2^60): the reciprocal and the root are the correctly rounded ones (IEEE operations of
-    numpy for two binades, of torch for the rest), and so are quotients by each of them, signs and a zero numerator included"""
+    numpy for two binades, of torch for the rest), and so is a quotient by each of them, signs and a zero numerator included
+    (numerators whose quotients lie next to a rounding boundary: test_quotient_rounding.py)"""
     import torch
     gen = torch.Generator("cuda").manual_seed(1)
     for exponent in range(67, 187, 4):
